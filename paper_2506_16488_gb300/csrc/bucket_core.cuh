@@ -1,0 +1,832 @@
+// Bucketed search kernel for graphs of low degree (road and grid shapes): one
+// CTA (team) runs a group of one or two searches to completion.
+//
+// Same algorithm as run_local (engine_core.cuh): Delta*-stepping buckets in
+// shared memory with lazy deletion, a far list beyond the ring's window, a
+// spill bitmap as the last resort.  What differs is the work of one step,
+// which on these graphs is short (100 to 500 entries) and bound by the chain
+// of dependent accesses and by instruction issue, not by bandwidth:
+//
+//  * Adjacency blocks: the first four edges of vertex v lie in one aligned
+//    block (GraphDev::blk16 / blk8: 64 bytes with the targets' potential
+//    coordinates, 32 without), so an entry needs neither its offsets nor a
+//    prefix sum over degrees: four lanes take one entry, lane q its q-th edge,
+//    and the block and the entry's distance are loaded together.  The chain is
+//    ring entry -> {block, own distance} -> target distance.  A vertex of more
+//    than four edges is inserted as two entries, so its continued edges are
+//    another entry's work, not a second pass of the same warp.
+//  * No potential at extraction: an entry's prune value is known from its
+//    bucket to within one step, and the stop rule (bk_decide) compares the
+//    bucket's smallest prune value with the bound, so testing each entry again
+//    would only save part of the last bucket.  The rule subtracts the key
+//    offset (h(s, t) for BiD-A*), which run_local's does not: it stops about
+//    12% of the steps earlier on the 1024^2 road graph.
+//  * The bucket index comes from a multiplication by a rounded-down reciprocal
+//    of the step, which gives the exact bucket or the one before it: an entry
+//    may be taken one step early, never late, and (b - 1) * step stays a lower
+//    bound of the keys in bucket b.
+//  * Positions in a bucket come from plain shared-memory atomics (78 cycles
+//    for 32 lanes on one address; a match of the lanes by bucket takes 99
+//    before its own atomic).
+//
+// Measured against run_local (which took 17,000 cycles a step for one query
+// alone on the GPU: decision 3,400, extraction 4,100, relaxation 6,900, the
+// rest waiting; an L2 hit takes 290-360): one BiD-A* query on the 1024^2 road
+// graph 7.3 -> 2.4 ms (4.6 -> 1.1 ms over random pairs, where the start ran
+// the whole GPU), 1,000 queries on it 45.5 -> 16.4 ms, 2,048 on the 2048^2
+// graph 228 -> 100 ms, 256 with 64-bit distances on the 4096^2 graph 255 ->
+// 136 ms.  DRAM traffic of the 2,048: 383 -> 213 GB.  What bounds it now: per
+// step and active warp about 500 instructions at 12.6 cycles each, of which a
+// third waits on global loads, a fifth on fixed-latency results and a seventh
+// on shared memory (one query alone); on a full GPU 0.46 of the issue slots
+// and 2.1 TB/s of random sectors, of the 1.95 TB/s that 155,000 independent
+// 4-byte loads from 1 GB reach.  Collecting the successful relaxations of the
+// CTA in shared memory, so that full warps take the second half, cut the
+// instructions but added a barrier per pass: 2,048 queries 100 -> 131 ms.
+#pragma once
+
+#include "engine_core.cuh"
+
+namespace ppsp {
+
+constexpr u32 BK_NB = 64;      // buckets in the ring (a power of two, two per lane of the deciding warp)
+constexpr u32 BK_DEFER = 64;   // entries with many edges handed to the whole CTA, per step
+constexpr u32 BK_QUAD_MAX = 32;  // continued edges that an entry's four lanes scan themselves
+constexpr u32 BK_EXTRA = 1u << 31;  // of a ring entry: the vertex's continued edges; of a target: it has some
+
+// Compiled variants of a group: BiDS and BiD-A* pairs, and single searches
+// (ET, A*, SSSP), which tell their mode apart at run time.
+enum { BK_BIDS = 0, BK_BIDASTAR = 1, BK_SINGLE = 2 };
+
+struct BkShared {
+    // the decision of a step, read by every thread
+    u64 cur, curkey;      // the bucket of the step and its threshold cur * step
+    u32 what, n, slot;    // what: 0 process bucket cur, 1 re-bucket far, 2 recover spills, 3 done
+    u32 late;             // 1 + largest (curkey - key) of the step's late entries, 0: none
+    u64 bound;            // prune bound: mu, or the largest target distance (SSSP)
+    u64 step;
+    i64 key_off;          // added to prune values to give keys (one value per group)
+    int2 pa, pb;          // anchors of search 0's potential: h_pb - h_pa (A*: h_pb)
+    u32 rn[BK_NB];
+    // far list: entries, smallest bucket, which of the slot's two arrays, and
+    // the entries right after the last re-bucketing
+    u32 far_n, far_at, far_after;
+    u64 far_min;
+    u32 tn, tov, spill, recov, idle;
+    u32 cnt_dir[2];       // stored entries per direction (pairs, kept while mu is unset)
+    u32 ndef;
+    SlotDev dev;          // the slot (its arrays are indexed at run time)
+    u32 src[2], sdir[2], pcnt[2];
+    PartnerDev pcache[2];
+    u32 group, flag;
+    u32 def_at[BK_DEFER], def_cnt[BK_DEFER], def_f[BK_DEFER];
+    u64 def_d[BK_DEFER];
+};
+
+__device__ __forceinline__ PartnerDev partner(const EngineArgs&, const BkShared& sm, u32 i, u32) { return sm.pcache[i]; }
+
+// A ring entry: flat index (BK_EXTRA), distance at insertion.
+template <typename D>
+struct BkEntry;
+template <>
+struct BkEntry<u32> {
+    typedef uint2 T;
+    static __device__ __forceinline__ T make(u32 f, u64 d) { return make_uint2(f, (u32)d); }
+};
+template <>
+struct BkEntry<u64> {
+    typedef ulonglong2 T;
+    static __device__ __forceinline__ T make(u32 f, u64 d) { return make_ulonglong2(f, d); }
+};
+
+template <typename D>
+constexpr size_t bucket_smem_bytes(u32 cap) {
+    return ((sizeof(BkShared) + 15) & ~(size_t)15) + (size_t)BK_NB * cap * sizeof(typename BkEntry<D>::T);
+}
+
+// One group's view: everything the inner functions need, in registers.
+template <typename D>
+struct BkCtx {
+    D* dist;
+    u32* touched;
+    typename BkEntry<D>::T* ring;
+    u32 cap, ob;  // shared-memory entries per bucket, entries of its overflow region
+    u32 tcap;
+    u32 mode, target, qe;
+    u32 d0, dm;   // direction of search i: d0 | (i & dm)
+    u32 magic;    // floor(2^32 / step)
+    u32 cur_lo;   // this step's bucket (low bits)
+    i64 kc;       // the group's key offset less that threshold: key - threshold = prune value + kc
+    u32 c_x, c_e, c_r, c_p, c_t;
+    int dc0, dc1;  // net change of the per-direction entry counts (pairs)
+};
+
+// mu <- min(mu, s); s is the length of a real path.
+template <typename D>
+__device__ __forceinline__ void bk_try_mu(const EngineArgs& a, const BkCtx<D>& c, BkShared& sm, u64 s) {
+    if (s >= sm.bound) return;
+    atomicMin(reinterpret_cast<unsigned long long*>(&sm.bound), (unsigned long long)s);
+    atomicMin(reinterpret_cast<unsigned long long*>(a.mu + c.qe), (unsigned long long)s);
+}
+
+// h_x(v) = floor(|P(v) - P(x)| / 2^F), exact: r with (r 2^F)^2 <= |P(v) - P(x)|^2
+// < ((r + 1) 2^F)^2, from a float32 estimate and integer comparisons.  The
+// estimate's relative error is below 2^-21 (the roundings of the differences,
+// the sum and the hardware root), a few units below 2^24; above, float64.
+// Coordinates are below 2^30 in magnitude, so differences fit 32 bits and the
+// square of (r + 1) 2^F 64.
+__device__ __forceinline__ float bk_h_est(int dx, int dy, float scale) {
+    const float fx = (float)dx, fy = (float)dy;
+    float y;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fx * fx + fy * fy));
+    return y * scale;
+}
+static __device__ __noinline__ u64 bk_h_big(u64 d2, u32 shift) { return (u64)sqrt((double)d2) >> shift; }
+__device__ __forceinline__ u32 bk_h_fix(int dx, int dy, float est, u32 shift) {
+    const u64 d2 = (u64)((i64)dx * dx) + (u64)((i64)dy * dy);
+    const u32 one = 1u << shift;
+    u32 R = (est < 16777216.f ? (u32)est : (u32)bk_h_big(d2, shift)) << shift;
+    while ((u64)R * R > d2) R -= one;
+    while ((u64)(R + one) * (R + one) <= d2) R += one;
+    return R >> shift;
+}
+
+// Prune value of <v, i> at distance d (Table 2); q = P(v).
+template <typename D, int KIND>
+__device__ __forceinline__ i64 bk_prune_value(const EngineArgs& a, const BkCtx<D>& c, const BkShared& sm, u32 i,
+                                              int2 q, u64 d) {
+    if (KIND == BK_BIDS) return 2 * (i64)d;
+    if (KIND == BK_SINGLE && c.mode != GM_ASTAR) return (i64)d;
+    const u32 F = a.g.pot_shift;
+    const float scale = __uint_as_float((127u - F) << 23);  // 2^-F
+    const int2 pb = sm.pb;
+    const int bx = q.x - pb.x, by = q.y - pb.y;
+    const float eb = bk_h_est(bx, by, scale);
+    if (KIND == BK_SINGLE) return (i64)d + (i64)bk_h_fix(bx, by, eb, F);
+    const int2 pa = sm.pa;
+    const int ax = q.x - pa.x, ay = q.y - pa.y;
+    const float ea = bk_h_est(ax, ay, scale);
+    const i64 rho = (i64)bk_h_fix(bx, by, eb, F) - (i64)bk_h_fix(ax, ay, ea, F);
+    return 2 * (i64)d + (i ? -rho : rho);
+}
+
+// Entry (f, d) at position pos of ring slot s: shared memory, then the
+// bucket's overflow region.
+template <typename D>
+__device__ __forceinline__ bool bk_place(const BkCtx<D>& c, const BkShared& sm, u32 s, u32 pos, u32 f, u64 d) {
+    if (pos < c.cap) {
+        c.ring[s * c.cap + pos] = BkEntry<D>::make(f, d);
+        return true;
+    }
+    pos -= c.cap;
+    if (pos >= c.ob) return false;
+    sm.dev.of[(size_t)s * c.ob + pos] = f;
+    reinterpret_cast<D*>(sm.dev.od)[(size_t)s * c.ob + pos] = (D)d;
+    return true;
+}
+
+template <typename D>
+__device__ __forceinline__ bool bk_place_far(const BkShared& sm, u32 fb, u32 pos, u32 f, u64 d) {
+    if (pos >= sm.dev.qcap) return false;
+    sm.dev.q[fb][pos] = f;
+    reinterpret_cast<D*>(sm.dev.fd[fb])[pos] = (D)d;
+    return true;
+}
+
+// An entry that found no room: its bit in the slot's spill bitmap.  It is
+// recovered later with both parts (and counted as another entry; a part that
+// was stored is then taken twice, which is harmless).  Returns 1 for a new bit.
+static __device__ __noinline__ u32 bk_spill(BkShared& sm, u32 f) {
+    const u32 bit = 1u << (f & 31u);
+    if (atomicOr(sm.dev.bm[0] + (f >> 5), bit) & bit) return 0;
+    sm.spill = 1;
+    return 1;
+}
+
+// Far entries: beyond the ring's window.
+template <typename D>
+__device__ __forceinline__ void bk_insert_far(BkShared& sm, u32 db, u32 f, u32 f0, u32 num, u64 d, bool& s0, bool& s1) {
+    const u32 pos = atomicAdd(&sm.far_n, num);
+    s0 = bk_place_far<D>(sm, sm.far_at, pos, f0, d);
+    if (num == 2) s1 = bk_place_far<D>(sm, sm.far_at, pos + 1, f | BK_EXTRA, d);
+    atomicMin(reinterpret_cast<unsigned long long*>(&sm.far_min), (unsigned long long)(sm.cur + db));
+}
+
+// F.Add of flat index f at distance d and prune value pv.  extra: 0 its first
+// edges, BK_EXTRA its continued ones, 2 both (two entries).
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_insert(BkCtx<D>& c, BkShared& sm, u32 f, u32 extra, i64 pv, u64 d) {
+    const i64 rk = pv + c.kc;  // key less the step's threshold
+    const u32 num = extra == 2 ? 2u : 1u, f0 = extra == BK_EXTRA ? (f | BK_EXTRA) : f;
+    u32 db;  // buckets ahead of the current one
+    if (rk <= 0) {
+        // already under the threshold: due at the next step; the bucket's
+        // lower bound does not hold for it, so its distance below the
+        // threshold is remembered
+        db = 1;
+        const u64 below = (u64)-rk + 1;
+        atomicMax(&sm.late, below >> 32 ? 0xFFFFFFFFu : (u32)below);
+    } else if (((u64)rk >> 32) == 0) {
+        db = __umulhi((u32)rk - 1u, c.magic) + 1u;
+    } else {
+        const u64 q = ((u64)rk - 1) / sm.step + 1;
+        db = q < 0x7FFFFFFFull ? (u32)q : 0x7FFFFFFFu;
+    }
+    bool s0, s1 = true;  // stored: the entry, and its second one
+    if (db < BK_NB) {
+        const u32 s = (c.cur_lo + db) & (BK_NB - 1);
+        const u32 pos = atomicAdd(&sm.rn[s], num);
+        s0 = bk_place<D>(c, sm, s, pos, f0, d);
+        if (num == 2) s1 = bk_place<D>(c, sm, s, pos + 1, f | BK_EXTRA, d);
+    } else {
+        bk_insert_far<D>(sm, db, f, f0, num, d, s0, s1);
+    }
+    ++c.c_p;
+    u32 num_in = (s0 && extra != BK_EXTRA) ? 1u : 0u;  // stored entries that count for their direction
+    if (!(s0 && s1)) num_in += bk_spill(sm, f);
+    if (KIND != BK_SINGLE) {
+        if (f & 1u) c.dc1 += num_in; else c.dc0 += num_in;
+    }
+}
+
+// Both searches' distances of v (pair), or the one search's.
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_load(const BkCtx<D>& c, u32 v, u64& x0, u64& x1) {
+    if (KIND != BK_SINGLE) {
+        ld_pair(c.dist, v, x0, x1);
+    } else {
+        x0 = ld_dist(c.dist + v);
+        x1 = DT<D>::INF;
+    }
+}
+
+struct BkRec {
+    u32 v, w;  // target (bit 31: it has continued edges), weight
+    int2 q;    // P(target)
+};
+
+// Record k of the adjacency blocks (or, at >= 4n, of the continued edges).
+template <int KIND>
+__device__ __forceinline__ BkRec bk_rec(const EngineArgs& a, bool pot, u32 dir, size_t k) {
+    BkRec r;
+    if (KIND == BK_BIDASTAR || (KIND == BK_SINGLE && pot)) {
+        const int4 x = __ldg((dir ? a.g.blk16_t : a.g.blk16) + k);
+        r.v = (u32)x.x;
+        r.w = (u32)x.y;
+        r.q = make_int2(x.z, x.w);
+    } else {
+        const uint2 x = __ldg((dir ? a.g.blk8_t : a.g.blk8) + k);
+        r.v = x.x;
+        r.w = x.y;
+        r.q = make_int2(0, 0);
+    }
+    return r;
+}
+
+// Relaxation along record r of entry <f, d>, given the target's distances
+// just read: they decide success (a concurrent smaller write only leaves a
+// stale entry behind, which extraction drops), so the write is not waited for.
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, u32 f, u64 d, const BkRec& r,
+                                         u64 x0, u64 x1) {
+    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    const u32 i = KS ? (f & 1u) : 0u;
+    const u64 nd = d + (u64)r.w;
+    ++c.c_e;
+    if (nd > DT<D>::MAXV) {
+        // a distance that does not fit, unless the entry should have been
+        // pruned (extraction does not test that)
+        const int2 qv = a.g.pc ? __ldg(a.g.pc + (f >> KS)) : make_int2(0, 0);
+        if (!pruned(bk_prune_value<D, KIND>(a, c, sm, i, qv, d), sm.bound)) atomicOr(a.err, ERRB_OVERFLOW);
+        return;
+    }
+    const u64 own = i ? x1 : x0, oth = i ? x0 : x1;
+    if (nd >= own) return;
+    const u32 v2 = r.v & ~BK_EXTRA, f2 = (v2 << KS) | i;
+    amin_dist(c.dist + f2, nd);
+    ++c.c_r;
+    // the position in the touched list is asked for here and used at the end
+    const bool fresh = own == DT<D>::INF;
+    u32 tpos = 0;
+    if (fresh) {
+        ++c.c_t;
+        tpos = atomicAdd(&sm.tn, 1u);
+    }
+    if (KIND != BK_SINGLE) {
+        if (oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, nd + oth);
+    } else if (v2 == c.target) {
+        bk_try_mu<D>(a, c, sm, nd);
+    }
+    const i64 pv = bk_prune_value<D, KIND>(a, c, sm, i, r.q, nd);
+    if (!pruned(pv, sm.bound)) bk_insert<D, KIND>(c, sm, f2, (r.v & BK_EXTRA) ? 2u : 0u, pv, nd);
+    if (fresh) {
+        if (tpos < c.tcap)
+            c.touched[tpos] = f2;
+        else
+            sm.tov = 1;
+    }
+}
+
+// Take the bucket's entries: four lanes each.
+template <typename D, int B, int KIND>
+__device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
+    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    const u32 t = threadIdx.x, q4 = t & 3u;
+    const u32 n = sm.n, s = sm.slot;
+    for (u32 e = t >> 2; e < n; e += B / 4) {
+        u32 f;
+        u64 dins;
+        if (e < c.cap) {
+            const typename BkEntry<D>::T x = c.ring[s * c.cap + e];
+            f = (u32)x.x;
+            dins = x.y;
+        } else {
+            f = __ldcg(sm.dev.of + (size_t)s * c.ob + (e - c.cap));
+            dins = ld_dist(reinterpret_cast<const D*>(sm.dev.od) + (size_t)s * c.ob + (e - c.cap));
+        }
+        const u32 extra = f & BK_EXTRA;
+        f &= ~BK_EXTRA;
+        const u32 v = f >> KS, i = KS ? (f & 1u) : 0u, dir = c.d0 | (i & c.dm);
+        u64 x0, x1;
+        bk_load<D, KIND>(c, v, x0, x1);
+        u32 rest = 0;   // continued edges after these four
+        size_t at = (size_t)v * 4 + q4;
+        if (extra) {
+            // the fourth record holds where the edges go on
+            at = (size_t)bk_rec<KIND>(a, pot, dir, (size_t)v * 4 + 3).w + q4;
+            const u32* off = dir ? a.g.off_t : a.g.off;
+            rest = __ldg(off + v + 1) - __ldg(off + v) - 3;
+            rest = rest > 4 ? rest - 4 : 0;
+        }
+        BkRec r = bk_rec<KIND>(a, pot, dir, at);
+        const u64 d = i ? x1 : x0;
+        if (KIND != BK_SINGLE && q4 == 0 && !extra) {
+            if (i) --c.dc1; else --c.dc0;  // the stored entry is consumed
+        }
+        if (d != dins) continue;  // stale: a smaller distance was inserted again
+        if (q4 == 0 && !extra) {
+            ++c.c_x;
+            const u64 oth = i ? x0 : x1;
+            if (KIND != BK_SINGLE && oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, d + oth);
+        }
+        if (r.v < BLK_MORE) {
+            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
+            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+        }
+        if (rest) {
+            bool mine = true;
+            if (rest > BK_QUAD_MAX) {
+                // many edges: for the whole CTA, after the step's barrier
+                // (ndef may pass BK_DEFER: the readers clamp it)
+                if (q4 == 0) {
+                    const u32 k = atomicAdd(&sm.ndef, 1u);
+                    if (k < BK_DEFER) {
+                        sm.def_at[k] = (u32)(at + 4);
+                        sm.def_cnt[k] = rest;
+                        sm.def_f[k] = f;
+                        sm.def_d[k] = d;
+                    } else {
+                        // no room: this lane scans them all
+                        for (u32 j = 0; j < rest; ++j) {
+                            r = bk_rec<KIND>(a, pot, dir, at + 4 + j);
+                            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
+                            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+                        }
+                    }
+                }
+                mine = false;
+            }
+            for (u32 j = q4; mine && j < rest; j += 4) {
+                at += 4;
+                r = bk_rec<KIND>(a, pot, dir, at);
+                bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
+                bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+            }
+        }
+    }
+}
+
+// Entries with many edges: the whole CTA shares each one's.
+template <typename D, int B, int KIND>
+__device__ __forceinline__ void bk_deferred(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
+    const u32 nd = min(sm.ndef, BK_DEFER);
+    for (u32 k = 0; k < nd; ++k) {
+        const u32 f = sm.def_f[k], i = KIND == BK_SINGLE ? 0u : (f & 1u);
+        const u64 d = sm.def_d[k];
+        for (u32 j = threadIdx.x; j < sm.def_cnt[k]; j += B) {
+            const BkRec r = bk_rec<KIND>(a, pot, c.d0 | (i & c.dm), (size_t)sm.def_at[k] + j);
+            u64 x0, x1;
+            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
+            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sm.ndef = 0;
+}
+
+// A far or spilled entry back into the ring (or the other far list): dropped
+// when stale (dins = INF: a spilled one, taken from its current distance with
+// both parts).
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_rebucket(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot, u32 f,
+                                            u64 dins) {
+    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    u32 extra = f & BK_EXTRA;
+    f &= ~BK_EXTRA;
+    const u32 v = f >> KS, i = KS ? (f & 1u) : 0u;
+    const u64 d = ld_dist(c.dist + f);
+    const int2 q = pot ? __ldg(a.g.pc + v) : make_int2(0, 0);
+    if (KIND != BK_SINGLE && !extra) {
+        if (i) --c.dc1; else --c.dc0;
+    }
+    if (d == DT<D>::INF || (dins != DT<D>::INF && d != dins)) return;
+    if (dins == DT<D>::INF) {
+        const u32* off = (c.d0 | (i & c.dm)) ? a.g.off_t : a.g.off;
+        if (__ldg(off + v + 1) - __ldg(off + v) > 4) extra = 2;
+    }
+    bk_insert<D, KIND>(c, sm, f, extra, bk_prune_value<D, KIND>(a, c, sm, i, q, d), d);
+}
+
+template <typename D, int B, int KIND>
+__device__ __forceinline__ void bk_redistribute(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
+    const u32 t = threadIdx.x, from = sm.far_at;
+    const u32 n = min(sm.far_n, sm.dev.qcap);
+    __syncthreads();
+    if (t == 0) {
+        sm.far_at = from ^ 1u;
+        sm.far_n = 0;
+        sm.far_min = INF64;
+    }
+    __syncthreads();
+    for (u32 k = t; k < n; k += B)
+        bk_rebucket<D, KIND>(a, c, sm, pot, __ldcg(sm.dev.q[from] + k),
+                             ld_dist(reinterpret_cast<const D*>(sm.dev.fd[from]) + k));
+    __syncthreads();
+    if (t == 0) sm.far_after = sm.far_n;
+}
+
+template <typename D, int B, int KIND>
+__device__ __forceinline__ void bk_recover(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot, u32 nwords) {
+    if (threadIdx.x == 0) sm.spill = 0;
+    __syncthreads();
+    for (u32 w = threadIdx.x; w < nwords; w += B) {
+        u32 bits = __ldcg(sm.dev.bm[0] + w);
+        if (!bits) continue;
+        // cleared before its entries are inserted again: one that spills once
+        // more sets its bit again
+        atomicAnd(sm.dev.bm[0] + w, ~bits);
+        while (bits) {
+            const u32 f = (w << 5) | (u32)(__ffs(bits) - 1);
+            bits &= bits - 1;
+            bk_rebucket<D, KIND>(a, c, sm, pot, f, DT<D>::INF);
+        }
+    }
+}
+
+// The next step, decided by the first warp (every lane computes the same).
+// fresh: the entry counts per direction are up to date.
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c, BkShared& sm, bool fresh) {
+    const u32 t = threadIdx.x;
+    const u64 cur = sm.cur, curkey = sm.curkey, bound = sm.bound, step = sm.step, fmin = sm.far_min;
+    const i64 koff = sm.key_off;
+    const u32 lo = (u32)cur, spill = sm.spill, late = sm.late, farn = sm.far_n;
+    const u32 n0 = sm.rn[(lo + 1 + t) & (BK_NB - 1)];
+    const u32 n1 = t < 31 ? sm.rn[(lo + 33 + t) & (BK_NB - 1)] : 0u;
+    const u32 m0 = __ballot_sync(0xffffffffu, n0 != 0), m1 = __ballot_sync(0xffffffffu, n1 != 0);
+    // buckets ahead of the current one: first non-empty one of the ring, and
+    // of the far list (FAR: none, or at least that many)
+    constexpr u32 FAR = 1u << 30;
+    const u32 k = m0 ? (u32)__ffs(m0) : (m1 ? 32u + (u32)__ffs(m1) : FAR);
+    const u32 kf = farn ? (fmin - cur < FAR ? (u32)(fmin - cur) : FAR) : FAR;
+    const u32 nn = __shfl_sync(0xffffffffu, m0 ? n0 : n1, (k - 1) & 31);
+    const u32 kn = min(k, kf);
+    // mu certificate: every stored entry has key > (next bucket - 1) * step
+    // (or is a late one), and its prune value is its key less its offset; once
+    // that reaches the bound every remaining entry would be pruned.  App. B: a
+    // pair of which one side ran dry before mu was set is disconnected.
+    bool stop;
+    if (bound != INF64) {
+        i64 ahead = (i64)((u64)(kn - 1) * step) + 1;  // smallest key left, less curkey
+        if (kn == 1 && late) ahead = late != 0xFFFFFFFFu ? 1 - (i64)late : -(i64)curkey;
+        stop = !spill && bound > 0 && (i64)curkey + ahead - koff >= (i64)bound;
+    } else {
+        stop = KIND != BK_SINGLE && fresh && (sm.cnt_dir[0] == 0 || sm.cnt_dir[1] == 0);
+    }
+    u32 what = 0, ahead = k;
+    if (stop) {
+        what = 3;
+    } else if (spill || k == FAR || (farn && (kf <= k || kf < BK_NB / 2 || farn > sm.dev.qcap / 2))) {
+        const bool none = k == FAR && !farn;
+        if (spill && (!sm.recov || none)) {
+            // recover spilled entries before they fall behind, at most once
+            // between two processed buckets
+            what = 2;
+        } else if (farn && (kf <= k || kf < BK_NB / 2 || (farn > sm.dev.qcap / 2 && farn > 2 * sm.far_after))) {
+            // far entries due soon, an empty ring, or a far list filling up
+            // with stale entries (re-bucketing drops them)
+            what = 1;
+        } else if (k == FAR) {
+            what = spill ? 2 : 3;
+        }
+    }
+    if (t == 0) {
+        if (what == 0) {
+            sm.n = min(nn, c.cap + c.ob);
+            sm.slot = (lo + k) & (BK_NB - 1);
+            sm.recov = 0;
+            sm.idle = 0;
+            sm.late = 0;  // late entries of this bucket's processing
+        } else {
+            // the window moves up to the far list's first bucket when the
+            // ring holds nothing before it
+            const u64 to = (what == 1 && (k == FAR || fmin - cur <= k) && fmin > cur + 1) ? fmin - 1 : cur;
+            ahead = 0;
+            sm.cur = to;
+            sm.curkey = curkey + (to - cur) * step;
+            if (what == 2) sm.recov = 1;
+            // a bounded number of decisions without a processed bucket: only
+            // an internal error gets here, never valid input
+            if (++sm.idle > 4096) {
+                atomicOr(a.err, ERRB_INTERNAL);
+                what = 3;
+            }
+        }
+        if (ahead) {
+            sm.cur = cur + ahead;
+            sm.curkey = curkey + (u64)ahead * step;
+        }
+        sm.what = what;
+    }
+}
+
+// Largest tentative distance of an SSSP group's targets (INF64 while one is
+// unreached), by one warp: prune bound and stop certificate (Sec. 4.3).
+template <typename D>
+__device__ __forceinline__ u64 bk_target_max(const EngineArgs& a, const BkCtx<D>& c, const GroupDev& G) {
+    u64 m = 0;
+    bool all = true;
+    for (u32 q = threadIdx.x & 31u; q < G.qcnt; q += 32) {
+        const u64 d = ld_dist(c.dist + a.qedges[G.qbeg + q].b);
+        all = all && d != DT<D>::INF;
+        m = d > m ? d : m;
+    }
+    all = __all_sync(0xffffffffu, all);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const u64 y = __shfl_xor_sync(0xffffffffu, m, o);
+        m = y > m ? y : m;
+    }
+    return (all && G.qcnt > 0) ? m : INF64;
+}
+
+// Add the warp's net entry counts per direction (pairs, while mu is unset:
+// they only serve the disconnected exit).
+template <typename D, int KIND>
+__device__ __forceinline__ void bk_flush_dir(BkCtx<D>& c, BkShared& sm) {
+    if (KIND == BK_SINGLE) return;
+    const u32 s0 = __reduce_add_sync(0xffffffffu, (u32)c.dc0);
+    const u32 s1 = __reduce_add_sync(0xffffffffu, (u32)c.dc1);
+    if ((threadIdx.x & 31) == 0) {
+        if (s0) atomicAdd(&sm.cnt_dir[0], s0);
+        if (s1) atomicAdd(&sm.cnt_dir[1], s1);
+    }
+    c.dc0 = c.dc1 = 0;
+}
+
+template <typename D, int B, int KIND>
+__device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const GroupDev& G, BkShared& sm,
+                                         unsigned char* ring) {
+    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    const u32 t = threadIdx.x;
+    const u64 t_start = (a.group_ns && t == 0) ? global_ns() : 0;
+    BkCtx<D> c;
+    c.dist = reinterpret_cast<D*>(sm.dev.dist);
+    c.touched = sm.dev.touched;
+    c.tcap = sm.dev.tcap;
+    c.cap = a.ring_cap;
+    c.ob = sm.dev.ocap / BK_NB;
+    c.ring = reinterpret_cast<typename BkEntry<D>::T*>(ring);
+    c.mode = G.mode;
+    c.target = G.target;
+    c.qe = G.qbeg;
+    c.c_x = c.c_e = c.c_r = c.c_p = c.c_t = 0;
+    c.dc0 = c.dc1 = 0;
+    const u32 flat_range = a.g.n << KS, nwords = (flat_range + 31u) >> 5;
+    const u64 step = KIND != BK_SINGLE ? 2 * G.delta : G.delta;
+    u32 sdeg = 0;
+    if (t < G.scnt) {
+        const SearchDev s = a.searches[G.sbeg + t];
+        const u32* off = s.dir ? a.g.off_t : a.g.off;
+        sdeg = __ldg(off + s.src + 1) - __ldg(off + s.src);
+        sm.src[t] = s.src;
+        sm.sdir[t] = s.dir;
+        sm.pcnt[t] = s.pcnt;
+        if (s.pcnt) sm.pcache[t] = a.partners[s.pbeg];
+        const u32 f = (s.src << KS) | t;
+        st_dist(c.dist + f, 0);
+        c.touched[t] = f;
+        if (t == 0) {
+            sm.key_off = s.key_off;
+            if (a.g.pc != nullptr) {
+                sm.pa = a.g.pc[s.src];
+                sm.pb = a.g.pc[s.pot_b];
+            }
+        }
+    }
+    if (t < BK_NB) sm.rn[t] = 0;
+    if (t == 0) {
+        sm.bound = INF64;
+        sm.step = step;
+        sm.cur = sm.curkey = 0;
+        sm.late = 0;
+        sm.far_n = sm.far_at = sm.far_after = 0;
+        sm.far_min = INF64;
+        sm.tn = G.scnt;
+        sm.tov = sm.spill = sm.recov = sm.idle = sm.ndef = 0;
+        sm.cnt_dir[0] = sm.cnt_dir[1] = 0;
+    }
+    for (u32 q = t; q < G.qcnt; q += B) a.mu[G.qbeg + q] = INF64;
+    __syncthreads();
+    const bool pot = KIND == BK_BIDASTAR || (KIND == BK_SINGLE && c.mode == GM_ASTAR);
+    c.d0 = KIND == BK_SINGLE ? sm.sdir[0] : 0u;
+    c.dm = KIND == BK_SINGLE ? 0u : sm.sdir[1];
+    c.magic = step > 1 ? (u32)((1ull << 32) / step) : 0xFFFFFFFFu;
+    c.cur_lo = 0;
+    c.kc = sm.key_off;
+    // Init: the sources (key 0) go to the first step
+    if (t < G.scnt) bk_insert<D, KIND>(c, sm, (sm.src[t] << KS) | t, sdeg > 4 ? 2u : 0u, -sm.key_off, 0);
+    bk_flush_dir<D, KIND>(c, sm);
+    __syncthreads();
+    u64 rounds = 0;
+    bool fresh = false;
+    for (;;) {
+        if (t < 32) bk_decide<D, KIND>(a, c, sm, fresh);
+        __syncthreads();
+        const u32 what = sm.what;
+        if (what == 3) break;
+        c.cur_lo = (u32)sm.cur;
+        c.kc = sm.key_off - (i64)sm.curkey;
+        fresh = false;
+        if (what == 0) {
+            bk_process<D, B, KIND>(a, c, sm, pot);
+            if (KIND == BK_SINGLE && c.mode == GM_SSSP && t >= B - 32 && (rounds & 3) == 0) {
+                __syncwarp();
+                const u64 m = bk_target_max<D>(a, c, G);
+                if (t == B - 32) atomicMin(reinterpret_cast<unsigned long long*>(&sm.bound), (unsigned long long)m);
+            }
+            ++rounds;
+        } else if (what == 1) {
+            bk_redistribute<D, B, KIND>(a, c, sm, pot);
+        } else {
+            bk_recover<D, B, KIND>(a, c, sm, pot, nwords);
+        }
+        __syncwarp();
+        if (KIND != BK_SINGLE && what == 0 && (rounds & 15) == 0) {
+            // the counts per direction only serve the disconnected exit,
+            // which may come some steps later
+            bk_flush_dir<D, KIND>(c, sm);
+            fresh = true;
+        }
+        if (what == 0 && t == 0) sm.rn[sm.slot] = 0;  // nothing is inserted into the processed bucket
+        __syncthreads();
+        if (what == 0 && sm.ndef) {
+            bk_deferred<D, B, KIND>(a, c, sm, pot);
+            fresh = false;
+            __syncthreads();
+        }
+    }
+    // entries left in the spill bitmap by an early stop
+    if (sm.spill)
+        for (u32 w = t; w < nwords; w += B) sm.dev.bm[0][w] = 0u;
+    if (KIND == BK_SINGLE && c.mode == GM_SSSP) {
+        for (u32 q = t; q < G.qcnt; q += B) {
+            const u64 d = ld_dist(c.dist + a.qedges[G.qbeg + q].b);
+            a.mu[G.qbeg + q] = (d == DT<D>::INF) ? INF64 : d;
+        }
+    }
+    const u32 tn = min(sm.tn, c.tcap);
+    const bool tov = sm.tov != 0;
+    if (a.path_buf != nullptr) {
+        __syncthreads();
+        TeamCtx tc{0, 0, 1, nullptr, false, 1};
+        GCtx<D> g;
+        g.G = G;
+        g.dist = c.dist;
+        g.n = a.g.n;
+        g.slot = sm.dev;
+        find_paths<D, B>(a, tc, g, sm, flat_range, tn, tov);
+    }
+    __syncthreads();
+    if (tov) {
+        for (u32 f = t; f < flat_range; f += B) st_dist(c.dist + f, DT<D>::INF);
+    } else {
+#pragma unroll 4
+        for (u32 k = t; k < tn; k += B) st_dist(c.dist + __ldcg(c.touched + k), DT<D>::INF);
+    }
+    if (a.counters) {
+        unsigned long long* cp = &a.counters->extracted;
+        const u32 mine[5] = {c.c_x, c.c_e, c.c_r, c.c_p, c.c_t};
+        const int at[5] = {0, 1, 2, 3, 7};
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            u64 x = mine[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            if ((t & 31u) == 0 && x) atomicAdd(cp + at[k], (unsigned long long)x);
+        }
+        if (t == 0) {
+            atomicAdd(cp + 4, (unsigned long long)rounds);
+            atomicAdd(cp + 5, 1ull);
+            atomicAdd(cp + 6, (unsigned long long)G.scnt);
+        }
+    }
+    if (a.group_ns && t == 0) a.group_ns[gi] = global_ns() - t_start;
+    __syncthreads();
+}
+
+// Threads per SM the kernel is compiled to keep resident (64 registers).
+template <int B>
+struct BucketMinBlocks {
+    static constexpr int value = 1024 / B;
+};
+
+// No CTA waits for another one, so the launch is an ordinary one: each CTA is
+// a team that takes groups from its queue.
+template <typename D, int B>
+__global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(EngineArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BkShared& sm = *reinterpret_cast<BkShared*>(smem_raw);
+    unsigned char* ring = smem_raw + ((sizeof(BkShared) + 15) & ~(size_t)15);
+    const u32 qid = a.team_queue[blockIdx.x];
+    if (threadIdx.x == 0) sm.dev = a.slots[blockIdx.x];
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const u32 idx = atomicAdd(a.queue_head + qid, 1u);
+            sm.group = idx < a.queue_len[qid] ? a.queue_items[qid][idx] : NONE;
+        }
+        __syncthreads();
+        const u32 gi = sm.group;
+        if (gi == NONE) break;
+        const GroupDev G = a.groups[gi];
+        if (G.mode != GM_BIDIR)
+            bk_group<D, B, BK_SINGLE>(a, gi, G, sm, ring);
+        else if (a.searches[G.sbeg].pot)
+            bk_group<D, B, BK_BIDASTAR>(a, gi, G, sm, ring);
+        else
+            bk_group<D, B, BK_BIDS>(a, gi, G, sm, ring);
+    }
+}
+
+// ---- host side ----
+constexpr size_t BK_SMEM_MAX = 227 * 1024;  // per CTA
+
+template <typename D, int B>
+static ppsp_status bucket_smem_attr() {
+    static std::atomic<bool> done[SMEM_ATTR_DEVICES];
+    int dev = 0;
+    PPSP_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < SMEM_ATTR_DEVICES && done[dev].load(std::memory_order_acquire)) return PPSP_OK;
+    PPSP_CUDA_TRY(cudaFuncSetAttribute(bucket_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)std::min<size_t>(bucket_smem_bytes<D>(RING_CAP_MAX), BK_SMEM_MAX)));
+    if (dev >= 0 && dev < SMEM_ATTR_DEVICES) done[dev].store(true, std::memory_order_release);
+    return PPSP_OK;
+}
+
+template <typename D, int B>
+static ppsp_status bucket_launch_t(const EngineArgs& a, u32 grid, cudaStream_t stream) {
+    ppsp_status st = bucket_smem_attr<D, B>();
+    if (st != PPSP_OK) return st;
+    bucket_kernel<D, B><<<grid, B, bucket_smem_bytes<D>(a.ring_cap), stream>>>(a);
+    PPSP_CUDA_TRY(cudaGetLastError());
+    return PPSP_OK;
+}
+
+template <typename D>
+static ppsp_status bucket_launch(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream) {
+    if (a.ring_cap < 1 || a.ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
+    if (block_threads == 256) return bucket_launch_t<D, 256>(a, grid, stream);
+    if (block_threads == 512) return bucket_launch_t<D, 512>(a, grid, stream);
+    if (block_threads == 1024) return bucket_launch_t<D, 1024>(a, grid, stream);
+    return PPSP_ERR_INVALID_ARG;
+}
+
+template <typename D, int B>
+static ppsp_status bucket_occ_t(int* bpsm, u32 ring_cap) {
+    ppsp_status st = bucket_smem_attr<D, B>();
+    if (st != PPSP_OK) return st;
+    PPSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, bucket_kernel<D, B>, B,
+                                                                bucket_smem_bytes<D>(ring_cap)));
+    return PPSP_OK;
+}
+
+template <typename D>
+static ppsp_status bucket_occ(int block_threads, u32 ring_cap, int* bpsm) {
+    if (ring_cap < 1 || ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
+    if (block_threads == 256) return bucket_occ_t<D, 256>(bpsm, ring_cap);
+    if (block_threads == 512) return bucket_occ_t<D, 512>(bpsm, ring_cap);
+    if (block_threads == 1024) return bucket_occ_t<D, 1024>(bpsm, ring_cap);
+    return PPSP_ERR_INVALID_ARG;
+}
+
+}  // namespace ppsp

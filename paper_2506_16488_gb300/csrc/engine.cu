@@ -13,26 +13,73 @@ ppsp_status engine_occupancy_u32(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u32_local(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64_local(int block_threads, u32 ring_cap, int* bpsm);
+// instantiated in bucket_{u32,u64}.cu
+ppsp_status launch_bucket_u32(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status launch_bucket_u64(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status bucket_occupancy_u32(int block_threads, u32 ring_cap, int* bpsm);
+ppsp_status bucket_occupancy_u64(int block_threads, u32 ring_cap, int* bpsm);
 
 ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
-                          cudaStream_t stream, bool local_only) {
-    if (dist_bits == 32)
-        return local_only ? launch_engine_u32_local(a, block_threads, grid, stream)
-                          : launch_engine_u32(a, block_threads, grid, stream);
-    return local_only ? launch_engine_u64_local(a, block_threads, grid, stream)
-                      : launch_engine_u64(a, block_threads, grid, stream);
+                          cudaStream_t stream, EngineKind kind) {
+    const bool w32 = dist_bits == 32;
+    if (kind == ENGINE_BUCKET)
+        return w32 ? launch_bucket_u32(a, block_threads, grid, stream) : launch_bucket_u64(a, block_threads, grid, stream);
+    if (kind == ENGINE_LOCAL)
+        return w32 ? launch_engine_u32_local(a, block_threads, grid, stream)
+                   : launch_engine_u64_local(a, block_threads, grid, stream);
+    return w32 ? launch_engine_u32(a, block_threads, grid, stream) : launch_engine_u64(a, block_threads, grid, stream);
 }
 
-ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms, bool local_only,
+ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms, EngineKind kind,
                              u32 ring_cap) {
     int dev = 0;
     PPSP_CUDA_TRY(cudaGetDevice(&dev));
     PPSP_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
-    if (dist_bits == 32)
-        return local_only ? engine_occupancy_u32_local(block_threads, ring_cap, blocks_per_sm)
-                          : engine_occupancy_u32(block_threads, ring_cap, blocks_per_sm);
-    return local_only ? engine_occupancy_u64_local(block_threads, ring_cap, blocks_per_sm)
-                      : engine_occupancy_u64(block_threads, ring_cap, blocks_per_sm);
+    const bool w32 = dist_bits == 32;
+    if (kind == ENGINE_BUCKET)
+        return w32 ? bucket_occupancy_u32(block_threads, ring_cap, blocks_per_sm)
+                   : bucket_occupancy_u64(block_threads, ring_cap, blocks_per_sm);
+    if (kind == ENGINE_LOCAL)
+        return w32 ? engine_occupancy_u32_local(block_threads, ring_cap, blocks_per_sm)
+                   : engine_occupancy_u64_local(block_threads, ring_cap, blocks_per_sm);
+    return w32 ? engine_occupancy_u32(block_threads, ring_cap, blocks_per_sm)
+               : engine_occupancy_u64(block_threads, ring_cap, blocks_per_sm);
+}
+
+// ---- adjacency blocks: one thread per record of a block; the thread of a
+// fourth record that continues writes the rest of the row ----
+__global__ void fill_blocks_kernel(const u32* off, const uint2* edges, const int4* edges_pc, const u32* more, u32 n,
+                                   uint2* blk8, int4* blk16) {
+    const u64 k = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+    const u64 v = k >> 2;
+    if (v >= n) return;
+    const u32 b0 = off[v], deg = off[v + 1] - b0, q = (u32)(k & 3);
+    const bool cont = deg > 4 && q == 3;
+    auto put = [&](u64 at, u32 e) {  // edge e, or an unused record
+        const uint2 none = make_uint2(BLK_NONE, 0u);
+        uint2 r = e < b0 + deg ? edges[e] : none;
+        int4 p = (blk16 && e < b0 + deg) ? edges_pc[e] : make_int4(0, 0, 0, 0);
+        if (e < b0 + deg && off[r.x + 1] - off[r.x] > 4) r.x |= 1u << 31;
+        if (blk8) blk8[at] = r;
+        if (blk16) blk16[at] = make_int4((int)r.x, (int)r.y, p.z, p.w);
+    };
+    if (!cont) {
+        put(k, b0 + q);
+        return;
+    }
+    const u32 at = more[v];
+    if (blk8) blk8[k] = make_uint2(BLK_MORE, at);
+    if (blk16) blk16[k] = make_int4((int)BLK_MORE, (int)at, 0, 0);
+    // deg - 3 records, padded to a multiple of four
+    for (u32 j = 0; j < (deg & ~3u); ++j) put((u64)at + j, b0 + 3 + j);
+}
+
+ppsp_status launch_fill_blocks(const u32* off, const uint2* edges, const int4* edges_pc, const u32* more, u32 n,
+                               uint2* blk8, int4* blk16) {
+    const u64 blocks = ((u64)n * 4 + 255) / 256;
+    fill_blocks_kernel<<<(u32)blocks, 256>>>(off, edges, edges_pc, more, n, blk8, blk16);
+    PPSP_CUDA_TRY(cudaGetLastError());
+    return PPSP_OK;
 }
 
 // ---- potential evaluation (for checks against the oracle) ----

@@ -45,6 +45,7 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "ppsp_internal.h"
@@ -1612,8 +1613,8 @@ __device__ u64 run_local(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 nword
 // delta_i[u] + w(u, x) = delta_i[x] (smallest u first), writing x0, ..., q_i to
 // out[start ..] while below cap.  Weights are >= 1, so delta_i strictly
 // decreases along the walk; every such u has an exact delta_i because x does.
-template <typename D, int B>
-__device__ u64 walk_back(const EngineArgs& a, GCtx<D>& c, const Smem<B>& sm, u32 x0, u32 i, u32* out,
+template <typename D, int B, typename SM>
+__device__ u64 walk_back(const EngineArgs& a, GCtx<D>& c, const SM& sm, u32 x0, u32 i, u32* out,
                          u64 cap, u64 start) {
     const u32 lane = threadIdx.x & 31;
     u32 x = x0;
@@ -1650,14 +1651,14 @@ __device__ u64 walk_back(const EngineArgs& a, GCtx<D>& c, const Smem<B>& sm, u32
     return idx - start;
 }
 
-template <typename D, int B>
-__device__ bool find_paths(const EngineArgs& a, const TeamCtx& tc, GCtx<D>& c, Smem<B>& sm, u32 flat_range) {
+// tn, tov: entries of the touched list, and whether it overflowed.
+template <typename D, int B, typename SM>
+__device__ bool find_paths(const EngineArgs& a, const TeamCtx& tc, GCtx<D>& c, SM& sm, u32 flat_range, u32 tn,
+                           bool tov) {
     const GroupDev& G = c.G;
     const u32 t = threadIdx.x;
     if (G.mode == GM_BIDIR) {
         // meeting vertex of each query edge: smallest v with delta_a[v] + delta_b[v] = mu
-        const u32 tn = ld_volatile(&c.slot.st->touched_n);
-        const bool tov = ld_volatile(&c.slot.st->touched_overflow) != 0;
         const u32 lim = tov ? flat_range : min(tn, c.slot.tcap);
         for (u32 k = tc.rank * B + t; k < lim; k += tc.size * B) {
             const u32 f = tov ? k : __ldcg(c.slot.touched + k);
@@ -2039,7 +2040,10 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
     }
 
     // ---- paths (optional), before the distances are reset ----
-    if (a.path_buf != nullptr && !find_paths<D, B>(a, tc, c, sm, flat_range)) return false;
+    if (a.path_buf != nullptr &&
+        !find_paths<D, B>(a, tc, c, sm, flat_range, ld_volatile(&slot.st->touched_n),
+                          ld_volatile(&slot.st->touched_overflow) != 0))
+        return false;
 
     // ---- tidy the slot ----
     if (exit_count > 0) {

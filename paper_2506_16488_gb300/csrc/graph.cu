@@ -240,7 +240,10 @@ SlotLayout slot_layout(int dist_bits, u64 flat_cap, u32 qcap, u32 tcap, bool mem
     const u64 words = (flat_cap + 31) / 32;
     auto al = [](u64 x) { return (x + 255) & ~255ull; };
     SlotLayout L;
-    L.ocap = std::max<u64>(32 * 256, flat_cap / 4) / 32 * 32;
+    // entries beyond the ring's shared-memory ones, split between its buckets:
+    // at least 4,096 each, so that a coarse increment on a small graph does
+    // not spill (a spilled bucket costs a scan of the slot's bitmap)
+    L.ocap = std::max<u64>(64 * 4096, flat_cap / 4) / 64 * 64;
     L.b_dist = al(flat_cap * W);
     L.b_bm = al(words * 4);
     L.b_q = al((u64)qcap * 4);
@@ -484,6 +487,7 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         cudaFree(g->d_pc);
         cudaFree(g->d_edges_pc);
         cudaFree(g->d_edges_t_pc);
+        cudaFree(g->d_blocks);
         return e == cudaErrorMemoryAllocation ? PPSP_ERR_OOM : PPSP_ERR_CUDA;
     };
     if ((ce = cudaMalloc(&g->d_off, (n + 1) * 4)) != cudaSuccess) return fail(ce, "cudaMalloc(off)");
@@ -494,10 +498,11 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         return fail(ce, "cudaMemcpy(edges)");
     info.device_bytes = (n + 1) * 4 + m * 8;
     std::vector<uint2> edt;  // transpose records (directed graphs)
+    std::vector<u32> offt;
     if (!info.undirected) {
         // transpose (in-edges, each row sorted by source): backward searches
         // from a target and path walks of forward searches follow it
-        std::vector<u32> offt(n + 1, 0);
+        offt.assign(n + 1, 0);
         for (u64 e = 0; e < m; ++e) ++offt[targets[e] + 1];
         for (u64 v = 0; v < n; ++v) offt[v + 1] += offt[v];
         std::vector<u32> fill(offt.begin(), offt.end() - 1);
@@ -552,6 +557,58 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
             info.device_bytes += m * 16;
         }
     }
+    // Adjacency blocks for the bucketed kernel: graphs of average degree at
+    // most BLOCK_MAX_DEG (road and grid shapes have 3.6 to 4).  They are left
+    // out, and plans run over the offsets, when they would take more than an
+    // eighth of the free device memory or a record index 32 bits.
+    constexpr u64 BLOCK_MAX_DEG = 6;
+    if (m <= BLOCK_MAX_DEG * n && n < (1ull << 29)) {
+        const u32 dirs = info.undirected ? 1 : 2;
+        std::vector<u32> more[2];  // record index of the continued edges, per direction
+        u64 recs[2] = {0, 0};
+        for (u32 d = 0; d < dirs; ++d) {
+            more[d].assign(n, 0);
+            u64 at = 4 * n;
+            for (u64 v = 0; v < n; ++v) {
+                const u64 deg = d ? offt[v + 1] - offt[v] : g->deg[v];
+                if (deg > 4) {
+                    more[d][v] = (u32)at;
+                    at += deg & ~3ull;  // deg - 3 records, padded to a multiple of four
+                }
+            }
+            recs[d] = at;
+        }
+        const u64 rb = coords ? 24 : 8;  // bytes per record: 8, and 16 with coordinates
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && (recs[0] + recs[1]) * rb <= free_b / 8 &&
+            std::max(recs[0], recs[1]) < (1ull << 32) &&
+            cudaMalloc(&g->d_blocks, (recs[0] + recs[1]) * rb + n * 4) == cudaSuccess) {
+            char* p = (char*)g->d_blocks;
+            if (coords) {
+                g->d_blk16 = (int4*)p;
+                if (dirs == 2) g->d_blk16_t = g->d_blk16 + recs[0];
+                p += (recs[0] + recs[1]) * 16;
+            }
+            g->d_blk8 = (uint2*)p;
+            if (dirs == 2) g->d_blk8_t = g->d_blk8 + recs[0];
+            u32* d_more = (u32*)(p + (recs[0] + recs[1]) * 8);
+            for (u32 d = 0; d < dirs; ++d) {
+                if ((ce = cudaMemcpy(d_more, more[d].data(), n * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
+                    return fail(ce, "cudaMemcpy(blocks)");
+                const ppsp_status st =
+                    launch_fill_blocks(d ? g->d_off_t : g->d_off, d ? g->d_edges_t : g->d_edges,
+                                       d ? g->d_edges_t_pc : g->d_edges_pc, d_more, (u32)n,
+                                       d ? g->d_blk8_t : g->d_blk8, d ? g->d_blk16_t : g->d_blk16);
+                if (st != PPSP_OK) return fail(cudaErrorUnknown, "fill_blocks");
+                if ((ce = cudaDeviceSynchronize()) != cudaSuccess) return fail(ce, "fill_blocks");
+            }
+            info.device_bytes += (recs[0] + recs[1]) * rb + n * 4;
+        }
+        cudaGetLastError();
+    }
+    size_t free_now = 0, total_mem = 0;
+    if (cudaMemGetInfo(&free_now, &total_mem) == cudaSuccess) g->device_mem = total_mem;
+    cudaGetLastError();
     *out = g.release();
     return PPSP_OK;
 }
@@ -568,6 +625,7 @@ void ppsp_graph_destroy(ppsp_graph* g) {
     cudaFree(g->d_pc);
     cudaFree(g->d_edges_pc);
     cudaFree(g->d_edges_t_pc);
+    cudaFree(g->d_blocks);
     cudaFree(g->d_scratch_u32);
     cudaFree(g->d_scratch_i64);
     cudaGetLastError();

@@ -46,6 +46,12 @@ struct ppsp_graph {
     ppsp::u32* d_off_t = nullptr;  // transpose of a directed graph (null when undirected)
     uint2* d_edges_t = nullptr;
     int2* d_pc = nullptr;
+    uint64_t device_mem = 0;       // total memory of the device
+    void* d_blocks = nullptr;      // adjacency blocks (GraphDev::blk8 ...), one allocation, or null
+    uint2* d_blk8 = nullptr;
+    uint2* d_blk8_t = nullptr;     // directed graphs
+    int4* d_blk16 = nullptr;       // graphs with coordinates
+    int4* d_blk16_t = nullptr;
     std::vector<int64_t> pc_host;  // 2n potential coordinates
     double pot_scale = 0.0;
     int pot_shift = 0;
@@ -73,6 +79,10 @@ struct ppsp_graph {
         g.pc = d_pc;
         g.edges_pc = d_edges_pc;
         g.edges_t_pc = d_edges_t_pc ? d_edges_t_pc : d_edges_pc;
+        g.blk8 = d_blk8;
+        g.blk8_t = d_blk8_t ? d_blk8_t : d_blk8;
+        g.blk16 = d_blk16;
+        g.blk16_t = d_blk16_t ? d_blk16_t : d_blk16;
         g.n = (ppsp::u32)n;
         g.pot_shift = (ppsp::u32)pot_shift;
         g.m = (ppsp::u32)m;

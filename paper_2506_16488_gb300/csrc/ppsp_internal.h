@@ -28,6 +28,11 @@ constexpr u32 NONE = ~0u;
 constexpr int KMAX = 64;          // searches per group (query-graph vertices)
 constexpr int MAX_QUEUES = 2;     // group queues: 0 = multi-search groups, 1 = pairs/singles
 
+// Targets that are no vertex (with blocks, ids are below 2^30), see
+// GraphDev::blk8.
+constexpr u32 BLK_NONE = ~0u;
+constexpr u32 BLK_MORE = ~0u - 1u;
+
 // Group modes (plug-ins of Table 2).
 enum : u32 {
     GM_BIDIR = 0,    // BiDS / BiD-A* / Multi-BiDS: searches joined by query edges
@@ -51,6 +56,18 @@ struct GraphDev {
     // random load; null otherwise
     const int4* edges_pc;
     const int4* edges_t_pc;
+    // adjacency blocks (graphs of low degree, else null): vertex v's first
+    // four edges in records 4v .. 4v+3, one aligned block.  Unused records
+    // have the target BLK_NONE; of a vertex with more than four edges the
+    // fourth has the target BLK_MORE and, as its weight, the index of the
+    // record at which its edges go on (behind the blocks, in rows padded to
+    // four).  Bit 31 of a target says that the target has more than four
+    // edges.  blk16: with P(target) (graphs with coordinates); _t: of the
+    // transpose
+    const uint2* blk8;
+    const uint2* blk8_t;
+    const int4* blk16;
+    const int4* blk16_t;
     u32 n;
     u32 pot_shift;        // F: h = isqrt(d2 >> 2F)
     u32 m;                // adjacency entries (bounds of checked builds)
@@ -185,16 +202,27 @@ void set_last_device_error(u32 err);
 // Detail text for an internal host-side inconsistency (printf format).
 void set_last_internal_error(const char* fmt, ...);
 
-// Launch the persistent engine.  dist_bits selects the distance width.
-ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
-                          cudaStream_t stream, bool local_only = false);
+// The kernel of a plan: teams of any size (queue / bitmap frontier), or one
+// CTA per team with buckets in shared memory, over the offsets (LOCAL) or over
+// the adjacency blocks of a graph of low degree (BUCKET: groups of one or two
+// searches).
+enum EngineKind { ENGINE_GENERAL = 0, ENGINE_LOCAL = 1, ENGINE_BUCKET = 2 };
 
-// Max resident CTAs of the engine for a block size / distance width (of the
-// one-CTA instance when local_only).
+// Launch a plan's kernel.  dist_bits selects the distance width.
+ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
+                          cudaStream_t stream, EngineKind kind = ENGINE_GENERAL);
+
+// Max resident CTAs of a kernel for a block size / distance width.
 // ring_cap: shared-memory entries per bucket of the one-CTA frontier.
 constexpr u32 RING_CAP_DEFAULT = 64;
 ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms,
-                             bool local_only = false, u32 ring_cap = RING_CAP_DEFAULT);
+                             EngineKind kind = ENGINE_GENERAL, u32 ring_cap = RING_CAP_DEFAULT);
+
+// Fill the adjacency blocks of one direction on the device (blk16 from
+// edges_pc, blk8 from edges; either may be null).  more[v]: record index of
+// the continued edges of vertex v (read for vertices of more than four edges).
+ppsp_status launch_fill_blocks(const u32* off, const uint2* edges, const int4* edges_pc, const u32* more, u32 n,
+                               uint2* blk8, int4* blk16);
 
 // Evaluate potentials h_anchor(v) on the device.
 ppsp_status launch_potential_eval(const GraphDev& g, u32 anchor, const u32* d_verts, u64 count,
