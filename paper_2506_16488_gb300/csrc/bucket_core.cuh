@@ -1,5 +1,6 @@
 // Bucketed search kernel for graphs of low degree (road and grid shapes): one
-// CTA (team) runs a group of one or two searches to completion.
+// CTA runs a group of one or two searches to completion, and a team of CTAs a
+// Multi-BiDS group, one search each (see bk_update).
 //
 // Same algorithm as run_local (engine_core.cuh): Delta*-stepping buckets in
 // shared memory with lazy deletion, a far list beyond the ring's window, a
@@ -54,9 +55,11 @@ constexpr u32 BK_DEFER = 64;   // entries with many edges handed to the whole CT
 constexpr u32 BK_QUAD_MAX = 32;  // continued edges that an entry's four lanes scan themselves
 constexpr u32 BK_EXTRA = 1u << 31;  // of a ring entry: the vertex's continued edges; of a target: it has some
 
-// Compiled variants of a group: BiDS and BiD-A* pairs, and single searches
-// (ET, A*, SSSP), which tell their mode apart at run time.
-enum { BK_BIDS = 0, BK_BIDASTAR = 1, BK_SINGLE = 2 };
+// Compiled variants: BiDS and BiD-A* pairs, single searches (ET, A*, SSSP),
+// which tell their mode apart at run time, and one search of a Multi-BiDS
+// group.  The last two are one search: their ring and lists hold vertices.
+enum { BK_BIDS = 0, BK_BIDASTAR = 1, BK_SINGLE = 2, BK_MULTI = 3 };
+constexpr bool bk_one(int kind) { return kind == BK_SINGLE || kind == BK_MULTI; }
 
 struct BkShared {
     // the decision of a step, read by every thread
@@ -79,6 +82,11 @@ struct BkShared {
     u32 src[2], sdir[2], pcnt[2];
     PartnerDev pcache[2];
     u32 group, flag;
+    // a Multi-BiDS search: its partners j, their query edges and mu (mirrors,
+    // never below a.mu); muj[j] = 0 where j is no partner
+    u32 pj[KMAX], npart;
+    u32 qej[KMAX];
+    u64 muj[KMAX];
     u32 def_at[BK_DEFER], def_cnt[BK_DEFER], def_f[BK_DEFER];
     u64 def_d[BK_DEFER];
 };
@@ -114,6 +122,7 @@ struct BkCtx {
     u32 tcap;
     u32 mode, target, qe;
     u32 d0, dm;   // direction of search i: d0 | (i & dm)
+    u32 ks, i0;   // one search of a group: its distances are dist[(v << ks) | i0]
     u32 magic;    // floor(2^32 / step)
     u32 cur_lo;   // this step's bucket (low bits)
     i64 kc;       // the group's key offset less that threshold: key - threshold = prune value + kc
@@ -155,7 +164,7 @@ __device__ __forceinline__ u32 bk_h_fix(int dx, int dy, float est, u32 shift) {
 template <typename D, int KIND>
 __device__ __forceinline__ i64 bk_prune_value(const EngineArgs& a, const BkCtx<D>& c, const BkShared& sm, u32 i,
                                               int2 q, u64 d) {
-    if (KIND == BK_BIDS) return 2 * (i64)d;
+    if (KIND == BK_BIDS || KIND == BK_MULTI) return 2 * (i64)d;
     if (KIND == BK_SINGLE && c.mode != GM_ASTAR) return (i64)d;
     const u32 F = a.g.pot_shift;
     const float scale = __uint_as_float((127u - F) << 23);  // 2^-F
@@ -244,7 +253,7 @@ __device__ __forceinline__ void bk_insert(BkCtx<D>& c, BkShared& sm, u32 f, u32 
     ++c.c_p;
     u32 num_in = (s0 && extra != BK_EXTRA) ? 1u : 0u;  // stored entries that count for their direction
     if (!(s0 && s1)) num_in += bk_spill(sm, f);
-    if (KIND != BK_SINGLE) {
+    if (!bk_one(KIND)) {
         if (f & 1u) c.dc1 += num_in; else c.dc0 += num_in;
     }
 }
@@ -252,12 +261,91 @@ __device__ __forceinline__ void bk_insert(BkCtx<D>& c, BkShared& sm, u32 f, u32 
 // Both searches' distances of v (pair), or the one search's.
 template <typename D, int KIND>
 __device__ __forceinline__ void bk_load(const BkCtx<D>& c, u32 v, u64& x0, u64& x1) {
-    if (KIND != BK_SINGLE) {
+    if (!bk_one(KIND)) {
         ld_pair(c.dist, v, x0, x1);
     } else {
-        x0 = ld_dist(c.dist + v);
+        x0 = ld_dist(c.dist + (KIND == BK_MULTI ? (((size_t)v << c.ks) | c.i0) : (size_t)v));
         x1 = DT<D>::INF;
     }
+}
+
+// Address of the distance of flat index f.
+template <typename D, int KIND>
+__device__ __forceinline__ D* bk_at(const BkCtx<D>& c, u32 f) {
+    return c.dist + (KIND == BK_MULTI ? (((size_t)f << c.ks) | c.i0) : (size_t)f);
+}
+
+// UpdateDistance of a Multi-BiDS search at vertex v, whose distance nd it has
+// just written.  The searches of a group run on CTAs of their own with no
+// barrier between them (each at its own threshold: Theorem 3.3 holds per query
+// for any schedule, and their frontiers grow at about the same rate).  Two
+// searches that write their final distances of v at the same time must not
+// miss each other: each writes with an atomic whose result it waits for, then
+// a fence, then reads the other's distance, so whichever write comes second
+// sees the first.  Nothing has to be read again at extraction.
+//
+// Measured (24-clique on the 1024^2 road graph, 11.8 M extractions): one team
+// of all CTAs on the queue / bitmap frontier, which inserts every waiting
+// entry again at every step, 244 ms; one CTA per search 41 ms (48 before the
+// row's loads were issued together; the fence is 8% of it), bound by the
+// latency of a step whose distances are a 128-byte row apart.
+template <typename D>
+__device__ __forceinline__ void bk_update_one(const EngineArgs& a, BkShared& sm, u32 j, u64 o, u64 nd) {
+    const u64 s = nd + o;
+    if (o != DT<D>::INF && s < sm.muj[j]) {
+        atomicMin(reinterpret_cast<unsigned long long*>(&sm.muj[j]), (unsigned long long)s);
+        atomicMin(reinterpret_cast<unsigned long long*>(a.mu + sm.qej[j]), (unsigned long long)s);
+    }
+}
+template <typename D>
+__device__ __forceinline__ void bk_update(const EngineArgs& a, const BkCtx<D>& c, BkShared& sm, u32 v, u64 nd) {
+    __threadfence();
+    const D* row = c.dist + ((size_t)v << c.ks);
+    const u32 np = sm.npart;
+    if (np <= 4) {
+        for (u32 p = 0; p < np; ++p) bk_update_one<D>(a, sm, sm.pj[p], ld_dist(row + sm.pj[p]), nd);
+        return;
+    }
+    // the whole row, 64 bytes in flight (a row has at least eight entries
+    // here); most of them are still infinite
+    constexpr u32 V = 16 / sizeof(D), CH = sizeof(D) == 4 ? 2 : 4;
+    for (u32 j0 = 0; j0 < (1u << c.ks); j0 += CH * V) {
+        uint4 x[CH];
+#pragma unroll
+        for (u32 k = 0; k < CH; ++k) x[k] = __ldcg(reinterpret_cast<const uint4*>(row + j0 + k * V));
+#pragma unroll
+        for (u32 k = 0; k < CH; ++k) {
+            const u32 j = j0 + k * V;
+            if ((x[k].x & x[k].y & x[k].z & x[k].w) == ~0u) continue;
+            if (sizeof(D) == 4) {
+                bk_update_one<D>(a, sm, j, x[k].x, nd);
+                bk_update_one<D>(a, sm, j + 1, x[k].y, nd);
+                bk_update_one<D>(a, sm, j + 2, x[k].z, nd);
+                bk_update_one<D>(a, sm, j + 3, x[k].w, nd);
+            } else {
+                bk_update_one<D>(a, sm, j, ((u64)x[k].y << 32) | x[k].x, nd);
+                bk_update_one<D>(a, sm, j + 1, ((u64)x[k].w << 32) | x[k].z, nd);
+            }
+        }
+    }
+}
+
+// Refresh a Multi-BiDS search's mirrors of mu and its prune bound, the
+// largest of them (mumax, Table 2), by one warp.
+__device__ __forceinline__ void bk_refresh(const EngineArgs& a, BkShared& sm) {
+    u64 m = 0;
+    for (u32 p = threadIdx.x & 31u; p < sm.npart; p += 32) {
+        const u32 j = sm.pj[p];
+        const u64 x = ldcg64(a.mu + sm.qej[j]);
+        atomicMin(reinterpret_cast<unsigned long long*>(&sm.muj[j]), (unsigned long long)x);
+        m = x > m ? x : m;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const u64 y = __shfl_xor_sync(0xffffffffu, m, o);
+        m = y > m ? y : m;
+    }
+    if ((threadIdx.x & 31u) == 0) atomicMin(reinterpret_cast<unsigned long long*>(&sm.bound), (unsigned long long)m);
 }
 
 struct BkRec {
@@ -289,7 +377,7 @@ __device__ __forceinline__ BkRec bk_rec(const EngineArgs& a, bool pot, u32 dir, 
 template <typename D, int KIND>
 __device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, u32 f, u64 d, const BkRec& r,
                                          u64 x0, u64 x1) {
-    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
     const u32 i = KS ? (f & 1u) : 0u;
     const u64 nd = d + (u64)r.w;
     ++c.c_e;
@@ -303,7 +391,12 @@ __device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkSha
     const u64 own = i ? x1 : x0, oth = i ? x0 : x1;
     if (nd >= own) return;
     const u32 v2 = r.v & ~BK_EXTRA, f2 = (v2 << KS) | i;
-    amin_dist(c.dist + f2, nd);
+    if (KIND == BK_MULTI) {
+        if (amin_dist(bk_at<D, KIND>(c, f2), nd) <= nd) return;
+        bk_update<D>(a, c, sm, v2, nd);
+    } else {
+        amin_dist(c.dist + f2, nd);
+    }
     ++c.c_r;
     // the position in the touched list is asked for here and used at the end
     const bool fresh = own == DT<D>::INF;
@@ -312,9 +405,9 @@ __device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkSha
         ++c.c_t;
         tpos = atomicAdd(&sm.tn, 1u);
     }
-    if (KIND != BK_SINGLE) {
+    if (!bk_one(KIND)) {
         if (oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, nd + oth);
-    } else if (v2 == c.target) {
+    } else if (KIND == BK_SINGLE && v2 == c.target) {
         bk_try_mu<D>(a, c, sm, nd);
     }
     const i64 pv = bk_prune_value<D, KIND>(a, c, sm, i, r.q, nd);
@@ -330,7 +423,7 @@ __device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkSha
 // Take the bucket's entries: four lanes each.
 template <typename D, int B, int KIND>
 __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
-    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
     const u32 t = threadIdx.x, q4 = t & 3u;
     const u32 n = sm.n, s = sm.slot;
     for (u32 e = t >> 2; e < n; e += B / 4) {
@@ -360,14 +453,14 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
         }
         BkRec r = bk_rec<KIND>(a, pot, dir, at);
         const u64 d = i ? x1 : x0;
-        if (KIND != BK_SINGLE && q4 == 0 && !extra) {
+        if (!bk_one(KIND) && q4 == 0 && !extra) {
             if (i) --c.dc1; else --c.dc0;  // the stored entry is consumed
         }
         if (d != dins) continue;  // stale: a smaller distance was inserted again
         if (q4 == 0 && !extra) {
             ++c.c_x;
             const u64 oth = i ? x0 : x1;
-            if (KIND != BK_SINGLE && oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, d + oth);
+            if (!bk_one(KIND) && oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, d + oth);
         }
         if (r.v < BLK_MORE) {
             bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
@@ -411,7 +504,7 @@ template <typename D, int B, int KIND>
 __device__ __forceinline__ void bk_deferred(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
     const u32 nd = min(sm.ndef, BK_DEFER);
     for (u32 k = 0; k < nd; ++k) {
-        const u32 f = sm.def_f[k], i = KIND == BK_SINGLE ? 0u : (f & 1u);
+        const u32 f = sm.def_f[k], i = bk_one(KIND) ? 0u : (f & 1u);
         const u64 d = sm.def_d[k];
         for (u32 j = threadIdx.x; j < sm.def_cnt[k]; j += B) {
             const BkRec r = bk_rec<KIND>(a, pot, c.d0 | (i & c.dm), (size_t)sm.def_at[k] + j);
@@ -430,13 +523,13 @@ __device__ __forceinline__ void bk_deferred(const EngineArgs& a, BkCtx<D>& c, Bk
 template <typename D, int KIND>
 __device__ __forceinline__ void bk_rebucket(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot, u32 f,
                                             u64 dins) {
-    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
+    constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
     u32 extra = f & BK_EXTRA;
     f &= ~BK_EXTRA;
     const u32 v = f >> KS, i = KS ? (f & 1u) : 0u;
-    const u64 d = ld_dist(c.dist + f);
+    const u64 d = ld_dist(bk_at<D, KIND>(c, f));
     const int2 q = pot ? __ldg(a.g.pc + v) : make_int2(0, 0);
-    if (KIND != BK_SINGLE && !extra) {
+    if (!bk_one(KIND) && !extra) {
         if (i) --c.dc1; else --c.dc0;
     }
     if (d == DT<D>::INF || (dins != DT<D>::INF && d != dins)) return;
@@ -511,7 +604,7 @@ __device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c
         if (kn == 1 && late) ahead = late != 0xFFFFFFFFu ? 1 - (i64)late : -(i64)curkey;
         stop = !spill && bound > 0 && (i64)curkey + ahead - koff >= (i64)bound;
     } else {
-        stop = KIND != BK_SINGLE && fresh && (sm.cnt_dir[0] == 0 || sm.cnt_dir[1] == 0);
+        stop = !bk_one(KIND) && fresh && (sm.cnt_dir[0] == 0 || sm.cnt_dir[1] == 0);
     }
     u32 what = 0, ahead = k;
     if (stop) {
@@ -584,7 +677,7 @@ __device__ __forceinline__ u64 bk_target_max(const EngineArgs& a, const BkCtx<D>
 // they only serve the disconnected exit).
 template <typename D, int KIND>
 __device__ __forceinline__ void bk_flush_dir(BkCtx<D>& c, BkShared& sm) {
-    if (KIND == BK_SINGLE) return;
+    if (bk_one(KIND)) return;
     const u32 s0 = __reduce_add_sync(0xffffffffu, (u32)c.dc0);
     const u32 s1 = __reduce_add_sync(0xffffffffu, (u32)c.dc1);
     if ((threadIdx.x & 31) == 0) {
@@ -594,12 +687,14 @@ __device__ __forceinline__ void bk_flush_dir(BkCtx<D>& c, BkShared& sm) {
     c.dc0 = c.dc1 = 0;
 }
 
+// One group, or (BK_MULTI) search `rank` of one.  Returns false when a wait of
+// the team ran out.
 template <typename D, int B, int KIND>
-__device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const GroupDev& G, BkShared& sm,
-                                         unsigned char* ring) {
-    constexpr u32 KS = KIND == BK_SINGLE ? 0u : 1u;
-    const u32 t = threadIdx.x;
-    const u64 t_start = (a.group_ns && t == 0) ? global_ns() : 0;
+__device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc, u32 gi, const GroupDev& G,
+                                         BkShared& sm, unsigned char* ring) {
+    constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
+    const u32 t = threadIdx.x, rank = KIND == BK_MULTI ? tc.rank : 0u;
+    const u64 t_start = (a.group_ns && t == 0 && rank == 0) ? global_ns() : 0;
     BkCtx<D> c;
     c.dist = reinterpret_cast<D*>(sm.dev.dist);
     c.touched = sm.dev.touched;
@@ -610,24 +705,28 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
     c.mode = G.mode;
     c.target = G.target;
     c.qe = G.qbeg;
+    c.ks = KIND == BK_MULTI ? G.kshift : 0u;
+    c.i0 = rank;
     c.c_x = c.c_e = c.c_r = c.c_p = c.c_t = 0;
     c.dc0 = c.dc1 = 0;
     const u32 flat_range = a.g.n << KS, nwords = (flat_range + 31u) >> 5;
     const u64 step = KIND != BK_SINGLE ? 2 * G.delta : G.delta;
+    const u32 scnt = KIND == BK_MULTI ? 1u : G.scnt;  // searches of this CTA
     u32 sdeg = 0;
-    if (t < G.scnt) {
-        const SearchDev s = a.searches[G.sbeg + t];
+    if (t < scnt) {
+        const SearchDev s = a.searches[G.sbeg + rank + t];
         const u32* off = s.dir ? a.g.off_t : a.g.off;
         sdeg = __ldg(off + s.src + 1) - __ldg(off + s.src);
         sm.src[t] = s.src;
         sm.sdir[t] = s.dir;
         sm.pcnt[t] = s.pcnt;
-        if (s.pcnt) sm.pcache[t] = a.partners[s.pbeg];
+        if (KIND != BK_MULTI && s.pcnt) sm.pcache[t] = a.partners[s.pbeg];
         const u32 f = (s.src << KS) | t;
-        st_dist(c.dist + f, 0);
+        st_dist(bk_at<D, KIND>(c, f), 0);
         c.touched[t] = f;
         if (t == 0) {
-            sm.key_off = s.key_off;
+            sm.key_off = KIND == BK_MULTI ? 0 : s.key_off;
+            sm.npart = s.pcnt;
             if (a.g.pc != nullptr) {
                 sm.pa = a.g.pc[s.src];
                 sm.pb = a.g.pc[s.pot_b];
@@ -635,6 +734,7 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
         }
     }
     if (t < BK_NB) sm.rn[t] = 0;
+    if (KIND == BK_MULTI && t < KMAX) sm.muj[t] = 0;
     if (t == 0) {
         sm.bound = INF64;
         sm.step = step;
@@ -642,20 +742,32 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
         sm.late = 0;
         sm.far_n = sm.far_at = sm.far_after = 0;
         sm.far_min = INF64;
-        sm.tn = G.scnt;
+        sm.tn = scnt;
         sm.tov = sm.spill = sm.recov = sm.idle = sm.ndef = 0;
         sm.cnt_dir[0] = sm.cnt_dir[1] = 0;
     }
-    for (u32 q = t; q < G.qcnt; q += B) a.mu[G.qbeg + q] = INF64;
+    if (rank == 0)
+        for (u32 q = t; q < G.qcnt; q += B) a.mu[G.qbeg + q] = INF64;
     __syncthreads();
+    if (KIND == BK_MULTI) {
+        const u32 pbeg = a.searches[G.sbeg + rank].pbeg;
+        for (u32 p = t; p < sm.npart; p += B) {
+            const PartnerDev pd = a.partners[pbeg + p];
+            sm.pj[p] = pd.j;
+            sm.qej[pd.j] = pd.qe;
+            sm.muj[pd.j] = INF64;
+        }
+        // every search's source distance and mu are in place
+        if (!team_sync(tc, a, &sm.flag)) return false;
+    }
     const bool pot = KIND == BK_BIDASTAR || (KIND == BK_SINGLE && c.mode == GM_ASTAR);
-    c.d0 = KIND == BK_SINGLE ? sm.sdir[0] : 0u;
-    c.dm = KIND == BK_SINGLE ? 0u : sm.sdir[1];
+    c.d0 = bk_one(KIND) ? sm.sdir[0] : 0u;
+    c.dm = bk_one(KIND) ? 0u : sm.sdir[1];
     c.magic = step > 1 ? (u32)((1ull << 32) / step) : 0xFFFFFFFFu;
     c.cur_lo = 0;
     c.kc = sm.key_off;
     // Init: the sources (key 0) go to the first step
-    if (t < G.scnt) bk_insert<D, KIND>(c, sm, (sm.src[t] << KS) | t, sdeg > 4 ? 2u : 0u, -sm.key_off, 0);
+    if (t < scnt) bk_insert<D, KIND>(c, sm, (sm.src[t] << KS) | t, sdeg > 4 ? 2u : 0u, -sm.key_off, 0);
     bk_flush_dir<D, KIND>(c, sm);
     __syncthreads();
     u64 rounds = 0;
@@ -675,6 +787,10 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
                 const u64 m = bk_target_max<D>(a, c, G);
                 if (t == B - 32) atomicMin(reinterpret_cast<unsigned long long*>(&sm.bound), (unsigned long long)m);
             }
+            if (KIND == BK_MULTI && t >= B - 32) {
+                __syncwarp();
+                bk_refresh(a, sm);
+            }
             ++rounds;
         } else if (what == 1) {
             bk_redistribute<D, B, KIND>(a, c, sm, pot);
@@ -682,7 +798,7 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
             bk_recover<D, B, KIND>(a, c, sm, pot, nwords);
         }
         __syncwarp();
-        if (KIND != BK_SINGLE && what == 0 && (rounds & 15) == 0) {
+        if (!bk_one(KIND) && what == 0 && (rounds & 15) == 0) {
             // the counts per direction only serve the disconnected exit,
             // which may come some steps later
             bk_flush_dir<D, KIND>(c, sm);
@@ -707,22 +823,27 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
     }
     const u32 tn = min(sm.tn, c.tcap);
     const bool tov = sm.tov != 0;
-    if (a.path_buf != nullptr) {
+    if (KIND != BK_MULTI && a.path_buf != nullptr) {
         __syncthreads();
-        TeamCtx tc{0, 0, 1, nullptr, false, 1};
+        TeamCtx one{0, 0, 1, nullptr, false, 1};
         GCtx<D> g;
         g.G = G;
         g.dist = c.dist;
         g.n = a.g.n;
         g.slot = sm.dev;
-        find_paths<D, B>(a, tc, g, sm, flat_range, tn, tov);
+        find_paths<D, B>(a, one, g, sm, flat_range, tn, tov);
     }
-    __syncthreads();
+    if (KIND == BK_MULTI) {
+        // the other searches read these distances until they end, too
+        if (!team_sync(tc, a, &sm.flag)) return false;
+    } else {
+        __syncthreads();
+    }
     if (tov) {
-        for (u32 f = t; f < flat_range; f += B) st_dist(c.dist + f, DT<D>::INF);
+        for (u32 f = t; f < flat_range; f += B) st_dist(bk_at<D, KIND>(c, f), DT<D>::INF);
     } else {
 #pragma unroll 4
-        for (u32 k = t; k < tn; k += B) st_dist(c.dist + __ldcg(c.touched + k), DT<D>::INF);
+        for (u32 k = t; k < tn; k += B) st_dist(bk_at<D, KIND>(c, __ldcg(c.touched + k)), DT<D>::INF);
     }
     if (a.counters) {
         unsigned long long* cp = &a.counters->extracted;
@@ -737,12 +858,13 @@ __device__ __forceinline__ void bk_group(const EngineArgs& a, u32 gi, const Grou
         }
         if (t == 0) {
             atomicAdd(cp + 4, (unsigned long long)rounds);
-            atomicAdd(cp + 5, 1ull);
-            atomicAdd(cp + 6, (unsigned long long)G.scnt);
+            if (rank == 0) atomicAdd(cp + 5, 1ull);
+            atomicAdd(cp + 6, (unsigned long long)scnt);
         }
     }
-    if (a.group_ns && t == 0) a.group_ns[gi] = global_ns() - t_start;
+    if (a.group_ns && t == 0 && rank == 0) a.group_ns[gi] = global_ns() - t_start;
     __syncthreads();
+    return true;
 }
 
 // Threads per SM the kernel is compiled to keep resident (64 registers).
@@ -751,81 +873,136 @@ struct BucketMinBlocks {
     static constexpr int value = 1024 / B;
 };
 
-// No CTA waits for another one, so the launch is an ordinary one: each CTA is
-// a team that takes groups from its queue.
-template <typename D, int B>
+// TEAMS = false: each CTA is a team that takes groups from its queue; no CTA
+// waits for another one, so the launch is an ordinary one.  TEAMS: some teams
+// have several CTAs and run Multi-BiDS groups, one search per CTA (a
+// cooperative launch: the CTAs of a team meet when a group starts and ends).
+template <typename D, int B, bool TEAMS>
 __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(EngineArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BkShared& sm = *reinterpret_cast<BkShared*>(smem_raw);
     unsigned char* ring = smem_raw + ((sizeof(BkShared) + 15) & ~(size_t)15);
-    const u32 qid = a.team_queue[blockIdx.x];
-    if (threadIdx.x == 0) sm.dev = a.slots[blockIdx.x];
+    TeamCtx tc;
+    tc.team = TEAMS ? a.cta_team[blockIdx.x] : blockIdx.x;
+    tc.rank = TEAMS ? blockIdx.x - a.team_first[tc.team] : 0u;
+    tc.size = TEAMS ? a.team_size[tc.team] : 1u;
+    tc.ts = a.tstate + tc.team;
+    tc.global_bar = tc.size > 1;
+    tc.expect = tc.size;
+    tc.wait_shift = 4;
+    const u32 qid = a.team_queue[tc.team];
+    if (threadIdx.x == 0) {
+        SlotDev s = a.slots[tc.team];
+        if (TEAMS && tc.size > 1) {
+            // this CTA's share of the slot's lists; its spill bitmap covers
+            // the vertices, and both bitmaps together hold one per search
+            // (n bits each, rounded up to words, of 2n per search)
+            const u32 r = tc.rank, k = tc.size;
+            s.ocap = s.ocap / k / BK_NB * BK_NB;
+            s.of += (size_t)r * s.ocap;
+            s.od = reinterpret_cast<D*>(s.od) + (size_t)r * s.ocap;
+            s.qcap /= k;
+            s.tcap /= k;
+            for (int x = 0; x < 2; ++x) {
+                s.q[x] += (size_t)r * s.qcap;
+                s.fd[x] = reinterpret_cast<D*>(s.fd[x]) + (size_t)r * s.qcap;
+            }
+            s.touched += (size_t)r * s.tcap;
+            s.bm[0] += (size_t)r * ((a.g.n + 31u) / 32u);
+        }
+        sm.dev = s;
+    }
     for (;;) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && tc.rank == 0) {
             const u32 idx = atomicAdd(a.queue_head + qid, 1u);
-            sm.group = idx < a.queue_len[qid] ? a.queue_items[qid][idx] : NONE;
+            const u32 g = idx < a.queue_len[qid] ? a.queue_items[qid][idx] : NONE;
+            if (TEAMS && tc.global_bar) tc.ts->group = g;
+            sm.group = g;
+        }
+        if (TEAMS && tc.global_bar) {
+            if (!team_sync(tc, a, &sm.flag)) break;
+            if (threadIdx.x == 0) sm.group = ld_volatile(&tc.ts->group);
         }
         __syncthreads();
         const u32 gi = sm.group;
         if (gi == NONE) break;
         const GroupDev G = a.groups[gi];
+        if (TEAMS && tc.global_bar) {
+            // the team meets when the group starts, when its searches end
+            // and (above) before the next one is claimed
+            if (tc.rank < G.scnt) {
+                if (!bk_group<D, B, BK_MULTI>(a, tc, gi, G, sm, ring)) break;
+            } else {
+                if (!team_sync(tc, a, &sm.flag) || !team_sync(tc, a, &sm.flag)) break;
+            }
+            if (!team_sync(tc, a, &sm.flag)) break;
+            continue;
+        }
         if (G.mode != GM_BIDIR)
-            bk_group<D, B, BK_SINGLE>(a, gi, G, sm, ring);
+            bk_group<D, B, BK_SINGLE>(a, tc, gi, G, sm, ring);
         else if (a.searches[G.sbeg].pot)
-            bk_group<D, B, BK_BIDASTAR>(a, gi, G, sm, ring);
+            bk_group<D, B, BK_BIDASTAR>(a, tc, gi, G, sm, ring);
         else
-            bk_group<D, B, BK_BIDS>(a, gi, G, sm, ring);
+            bk_group<D, B, BK_BIDS>(a, tc, gi, G, sm, ring);
     }
 }
 
 // ---- host side ----
 constexpr size_t BK_SMEM_MAX = 227 * 1024;  // per CTA
 
-template <typename D, int B>
+template <typename D, int B, bool TEAMS>
 static ppsp_status bucket_smem_attr() {
     static std::atomic<bool> done[SMEM_ATTR_DEVICES];
     int dev = 0;
     PPSP_CUDA_TRY(cudaGetDevice(&dev));
     if (dev >= 0 && dev < SMEM_ATTR_DEVICES && done[dev].load(std::memory_order_acquire)) return PPSP_OK;
-    PPSP_CUDA_TRY(cudaFuncSetAttribute(bucket_kernel<D, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PPSP_CUDA_TRY(cudaFuncSetAttribute(bucket_kernel<D, B, TEAMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)std::min<size_t>(bucket_smem_bytes<D>(RING_CAP_MAX), BK_SMEM_MAX)));
     if (dev >= 0 && dev < SMEM_ATTR_DEVICES) done[dev].store(true, std::memory_order_release);
     return PPSP_OK;
 }
 
-template <typename D, int B>
+template <typename D, int B, bool TEAMS>
 static ppsp_status bucket_launch_t(const EngineArgs& a, u32 grid, cudaStream_t stream) {
-    ppsp_status st = bucket_smem_attr<D, B>();
+    ppsp_status st = bucket_smem_attr<D, B, TEAMS>();
     if (st != PPSP_OK) return st;
-    bucket_kernel<D, B><<<grid, B, bucket_smem_bytes<D>(a.ring_cap), stream>>>(a);
-    PPSP_CUDA_TRY(cudaGetLastError());
+    const size_t smem = bucket_smem_bytes<D>(a.ring_cap);
+    if (TEAMS) {
+        EngineArgs args = a;
+        void* params[] = {&args};
+        PPSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bucket_kernel<D, B, TEAMS>, dim3(grid), dim3(B), params,
+                                                  smem, stream));
+    } else {
+        bucket_kernel<D, B, TEAMS><<<grid, B, smem, stream>>>(a);
+        PPSP_CUDA_TRY(cudaGetLastError());
+    }
     return PPSP_OK;
 }
 
-template <typename D>
+template <typename D, bool TEAMS>
 static ppsp_status bucket_launch(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream) {
     if (a.ring_cap < 1 || a.ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
-    if (block_threads == 256) return bucket_launch_t<D, 256>(a, grid, stream);
-    if (block_threads == 512) return bucket_launch_t<D, 512>(a, grid, stream);
-    if (block_threads == 1024) return bucket_launch_t<D, 1024>(a, grid, stream);
+    if (block_threads == 256) return bucket_launch_t<D, 256, TEAMS>(a, grid, stream);
+    if (block_threads == 512) return bucket_launch_t<D, 512, TEAMS>(a, grid, stream);
+    if (block_threads == 1024) return bucket_launch_t<D, 1024, TEAMS>(a, grid, stream);
     return PPSP_ERR_INVALID_ARG;
 }
 
-template <typename D, int B>
+template <typename D, int B, bool TEAMS>
 static ppsp_status bucket_occ_t(int* bpsm, u32 ring_cap) {
-    ppsp_status st = bucket_smem_attr<D, B>();
+    ppsp_status st = bucket_smem_attr<D, B, TEAMS>();
     if (st != PPSP_OK) return st;
-    PPSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, bucket_kernel<D, B>, B,
+    PPSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, bucket_kernel<D, B, TEAMS>, B,
                                                                 bucket_smem_bytes<D>(ring_cap)));
     return PPSP_OK;
 }
 
-template <typename D>
+template <typename D, bool TEAMS>
 static ppsp_status bucket_occ(int block_threads, u32 ring_cap, int* bpsm) {
     if (ring_cap < 1 || ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
-    if (block_threads == 256) return bucket_occ_t<D, 256>(bpsm, ring_cap);
-    if (block_threads == 512) return bucket_occ_t<D, 512>(bpsm, ring_cap);
-    if (block_threads == 1024) return bucket_occ_t<D, 1024>(bpsm, ring_cap);
+    if (block_threads == 256) return bucket_occ_t<D, 256, TEAMS>(bpsm, ring_cap);
+    if (block_threads == 512) return bucket_occ_t<D, 512, TEAMS>(bpsm, ring_cap);
+    if (block_threads == 1024) return bucket_occ_t<D, 1024, TEAMS>(bpsm, ring_cap);
     return PPSP_ERR_INVALID_ARG;
 }
 

@@ -13,17 +13,24 @@ ppsp_status engine_occupancy_u32(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u32_local(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64_local(int block_threads, u32 ring_cap, int* bpsm);
-// instantiated in bucket_{u32,u64}.cu
+// instantiated in bucket_{u32,u64}{,_teams}.cu
 ppsp_status launch_bucket_u32(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
 ppsp_status launch_bucket_u64(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
-ppsp_status bucket_occupancy_u32(int block_threads, u32 ring_cap, int* bpsm);
-ppsp_status bucket_occupancy_u64(int block_threads, u32 ring_cap, int* bpsm);
+ppsp_status launch_bucket_u32_teams(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status launch_bucket_u64_teams(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status occupancy_bucket_u32(int block_threads, u32 ring_cap, int* bpsm);
+ppsp_status occupancy_bucket_u64(int block_threads, u32 ring_cap, int* bpsm);
+ppsp_status occupancy_bucket_u32_teams(int block_threads, u32 ring_cap, int* bpsm);
+ppsp_status occupancy_bucket_u64_teams(int block_threads, u32 ring_cap, int* bpsm);
 
 ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
                           cudaStream_t stream, EngineKind kind) {
     const bool w32 = dist_bits == 32;
     if (kind == ENGINE_BUCKET)
         return w32 ? launch_bucket_u32(a, block_threads, grid, stream) : launch_bucket_u64(a, block_threads, grid, stream);
+    if (kind == ENGINE_BUCKET_TEAMS)
+        return w32 ? launch_bucket_u32_teams(a, block_threads, grid, stream)
+                   : launch_bucket_u64_teams(a, block_threads, grid, stream);
     if (kind == ENGINE_LOCAL)
         return w32 ? launch_engine_u32_local(a, block_threads, grid, stream)
                    : launch_engine_u64_local(a, block_threads, grid, stream);
@@ -37,8 +44,11 @@ ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_s
     PPSP_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
     const bool w32 = dist_bits == 32;
     if (kind == ENGINE_BUCKET)
-        return w32 ? bucket_occupancy_u32(block_threads, ring_cap, blocks_per_sm)
-                   : bucket_occupancy_u64(block_threads, ring_cap, blocks_per_sm);
+        return w32 ? occupancy_bucket_u32(block_threads, ring_cap, blocks_per_sm)
+                   : occupancy_bucket_u64(block_threads, ring_cap, blocks_per_sm);
+    if (kind == ENGINE_BUCKET_TEAMS)
+        return w32 ? occupancy_bucket_u32_teams(block_threads, ring_cap, blocks_per_sm)
+                   : occupancy_bucket_u64_teams(block_threads, ring_cap, blocks_per_sm);
     if (kind == ENGINE_LOCAL)
         return w32 ? engine_occupancy_u32_local(block_threads, ring_cap, blocks_per_sm)
                    : engine_occupancy_u64_local(block_threads, ring_cap, blocks_per_sm);

@@ -135,6 +135,7 @@ struct TeamCtx {
     TeamState* ts;
     bool global_bar;  // size > 1 or a test hook forces the global path
     u32 expect;       // arrivals that release the barrier
+    u32 wait_shift = 0;  // spins allowed: the limit times 2^wait_shift (waits for a whole search)
 };
 
 static __device__ bool team_sync(const TeamCtx& tc, const EngineArgs& a, u32* s_flag) {
@@ -156,7 +157,7 @@ static __device__ bool team_sync(const TeamCtx& tc, const EngineArgs& a, u32* s_
                     ok = 0;
                     break;
                 }
-                if (++it > a.spin_limit) {
+                if (++it >> tc.wait_shift > a.spin_limit) {
                     atomicOr(a.err, ERRB_TIMEOUT);
                     ok = 0;
                     break;

@@ -787,16 +787,26 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     const u32 grid_max = grid;  // resident CTAs of the general kernel
 
     // ---- kernel ----
-    // Groups of one or two searches on a graph with adjacency blocks run the
+    // On a graph with adjacency blocks, groups of one or two searches run the
     // bucketed kernel, one CTA each, however few they are (the step of such a
     // group has a few hundred entries, which one CTA takes in less time than
-    // several need to meet at a barrier).  What that kernel does not do stays
-    // with the others: groups of more searches, explicit teams of several
-    // CTAs, a forced frontier, merged buckets (rho), memoized potentials, the
-    // pull step and the barrier test hook.
+    // several need to meet at a barrier), and larger groups run one CTA per
+    // search.  What that kernel does not do stays with the others: explicit
+    // team sizes, a forced frontier or layout, merged buckets (rho), memoized
+    // potentials, the pull step, multi-target potentials, paths of larger
+    // groups and the barrier test hook.
     const bool plain_opts = o.frontier == PPSP_FRONTIER_AUTO && o.debug_flags == 0;
-    if (plain_opts && big.empty() && g->d_blk8 && o.team_ctas <= 1 && !o.stepping_rho && !P->memo &&
-        !(o.pull_push && g->info.undirected)) {
+    bool bucket = plain_opts && g->d_blk8 && o.team_ctas <= 1 && !o.stepping_rho && !P->memo &&
+                  !(o.pull_push && g->info.undirected);
+    u32 tsize = 0;  // CTAs of a team for the larger groups: the most searches of one
+    for (u32 gi : big) {
+        tsize = std::max(tsize, P->groups[gi].scnt);
+        bucket = bucket && P->groups[gi].layout == PPSP_LAYOUT_INTERLEAVED;
+    }
+    if (tsize && (o.big_team_ctas || o.multi_potential || o.want_paths || strategy == PPSP_BATCH_PLAIN)) bucket = false;
+    if (bucket) {
+        const EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
+        const u64 want = small.size() + (u64)tsize * big.size();  // CTAs that run everything at once
         int bb = o.block_threads;
         if (!bb) {
             // Two groups per SM (512 threads each) when there are enough of
@@ -809,21 +819,37 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             for (u32 gi : small) range = std::max<u64>(range, n << P->groups[gi].kshift);
             const SlotCaps sc = slot_caps(range, o.frontier, false);
             const u64 two = 2ull * sms * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap);
-            bb = (small.size() > 4 * (size_t)sms && two <= g->device_mem / 4) ? 512 : 1024;
+            bb = (want > 4 * (u64)sms && two <= g->device_mem / 4) ? 512 : 1024;
         }
         const u32 cap = o.ring_entries ? o.ring_entries : bucket_cap(bb, o.dist_bits);
         int bbpsm = 0, bsms = 0;
-        st = engine_occupancy(o.dist_bits, bb, &bbpsm, &bsms, ENGINE_BUCKET, cap);
+        st = engine_occupancy(o.dist_bits, bb, &bbpsm, &bsms, kind, cap);
         if (st != PPSP_OK) return st;
-        if (bbpsm >= 1) {
-            grid = (u32)(bbpsm * bsms);
-            if (o.max_ctas > 0) grid = std::min<u32>(grid, (u32)o.max_ctas);
-            grid = strategy == PPSP_BATCH_PLAIN ? 1 : std::max<u32>(1, std::min<u32>(grid, (u32)small.size()));
-            teams.assign(grid, {1, 1});
-            P->queue_items[0].clear();
+        u32 res = (u32)(bbpsm * bsms);
+        if (o.max_ctas > 0) res = std::min<u32>(res, (u32)o.max_ctas);
+        // teams for the larger groups: one each when everything fits, else
+        // by their share of the estimated work
+        u32 nbt = 0;
+        if (tsize) {
+            double wb = 0, ws = 0;
+            for (u32 gi : big) wb += gwork[gi];
+            for (u32 gi : small) ws += gwork[gi];
+            const u32 room = small.empty() ? res : res - std::min<u32>(res, 1);
+            nbt = want <= res ? (u32)big.size()
+                              : std::min<u32>((u32)big.size(),
+                                              std::max<u32>(1, std::min<u32>(room, (u32)(res * wb / (wb + ws))) / tsize));
+        }
+        if (bbpsm >= 1 && res >= 1 && (u64)nbt * tsize + (small.empty() ? 0 : 1) <= res) {
+            const u32 left = res - nbt * tsize;
+            const u32 ns = small.empty() ? (tsize ? 0u : 1u)
+                                         : (strategy == PPSP_BATCH_PLAIN ? 1u : std::min<u32>(left, (u32)small.size()));
+            teams.assign(nbt, {tsize, 0});
+            teams.insert(teams.end(), ns, {1, 1});
+            grid = nbt * tsize + ns;
+            P->queue_items[0] = big;
             P->queue_items[1] = small;
             P->block = bb;
-            P->kind = ENGINE_BUCKET;
+            P->kind = kind;
             ring_cap = cap;
         }
     }

@@ -203,10 +203,11 @@ void set_last_device_error(u32 err);
 void set_last_internal_error(const char* fmt, ...);
 
 // The kernel of a plan: teams of any size (queue / bitmap frontier), or one
-// CTA per team with buckets in shared memory, over the offsets (LOCAL) or over
-// the adjacency blocks of a graph of low degree (BUCKET: groups of one or two
-// searches).
-enum EngineKind { ENGINE_GENERAL = 0, ENGINE_LOCAL = 1, ENGINE_BUCKET = 2 };
+// CTA per team with buckets in shared memory over the offsets (LOCAL), or the
+// same over the adjacency blocks of a graph of low degree: one CTA per group
+// of one or two searches (BUCKET), and one CTA per search of larger groups
+// (BUCKET_TEAMS).
+enum EngineKind { ENGINE_GENERAL = 0, ENGINE_LOCAL = 1, ENGINE_BUCKET = 2, ENGINE_BUCKET_TEAMS = 3 };
 
 // Launch a plan's kernel.  dist_bits selects the distance width.
 ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,

@@ -108,3 +108,31 @@ def test_disconnected_pairs_and_width_limit():
         assert st == ppsp.ERR_OVERFLOW
         got = G.batch(np.array([[0, 7], [22, 29]], dtype=np.uint32), mode="bids", strategy="plain_star")
         assert got.tolist() == [7 * w, 7 * w]
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("shape", ["clique3", "clique9", "star64", "mixed"])
+def test_groups_of_several_searches(shape, bits):
+    g, pairs = hub_graph(3000, DEGREES, seed=35, extra=4)
+    rng = np.random.default_rng(36)
+
+    def clique(k):
+        v = rng.choice(3000, k, replace=False)
+        i, j = np.triu_indices(k, 1)
+        return np.stack([v[i], v[j]], 1)
+
+    v = rng.choice(3000, 65, replace=False)
+    star = np.stack([np.full(63, v[0]), v[1:64]], 1)
+    p = {"clique3": clique(3), "clique9": clique(9), "star64": star,
+         "mixed": np.concatenate([pairs, clique(5), clique(3), star, [[3001, 1], [1, 17], [17, 3002]]])}[shape]
+    p = p.astype(np.uint32)
+    d = one_way_graph(g, 0.3, seed=37)
+    for graph, directed in ((g, False), (d, True)):
+        want = oracle.pairs(graph.offsets, graph.targets, graph.weights, p)
+        with ppsp.Graph.from_csr(graph, undirected=not directed) as G:
+            for mode in ("bids", "bidastar"):
+                for kw in ({}, {"delta": 30}, {"delta": 1 << 40, "ring_entries": 1}, {"block_threads": 512},
+                           {"block_threads": 256, "max_ctas": 66}, {"max_ctas": 2}):
+                    for _ in range(2):  # the second batch finds the slots as the first left them
+                        got = G.batch(p, mode=mode, strategy="multi", dist_bits=bits, **kw)
+                        assert np.array_equal(got, want), (directed, mode, kw)
