@@ -355,6 +355,7 @@ struct GCtx {
     u32* bm_nxt;
     u32* q_nxt;
     StepState* S_nxt;
+    StepState* S_cur;
     SlotDev slot;
     u64 theta;
     bool dense_nxt;
@@ -652,6 +653,33 @@ __device__ __forceinline__ void flush_stage(GCtx<D>& c, Smem<B>& sm) {
     __syncthreads();
 }
 
+// End of the part of row [b0, b1) worth scanning from distance d: with rows
+// sorted by weight, the first edge whose candidate d + w is above the prune
+// bound (mu for searches joined by query edges, not mu / 2: a candidate of
+// that length can still be the middle edge of a path).  A longer candidate
+// can neither lower mu nor be inserted.  A row whose last candidate does not
+// fit the width keeps its full length, so that the overflow is reported.
+// On RMAT graphs most weights exceed what is left of the bound: RMAT-20, one
+// BiDS query 55.8 -> 10.2 M edges, the batch of 75 single-source groups 10.2 ->
+// 3.4 G.
+template <typename D, int B>
+__device__ __forceinline__ u32 cut_row(const EngineArgs& a, const Smem<B>& sm, u32 i, u64 d, u32 b0, u32 b1) {
+    const u64 bound = sm.bound[i];
+    if (!a.g.wsorted || bound == INF64 || b1 - b0 < 2) return b1;
+    const uint2* ed = adj<B>(a, sm, i);
+    const u64 last = d + __ldg(&ed[b1 - 1].y);
+    if (last <= bound || last > DT<D>::MAXV) return b1;
+    u32 lo = b0, hi = b1 - 1;  // the first edge above the bound is in [lo, hi]
+    while (lo < hi) {
+        const u32 mid = lo + ((hi - lo) >> 1);
+        if (d + __ldg(&ed[mid].y) > bound)
+            hi = mid;
+        else
+            lo = mid + 1;
+    }
+    return lo;
+}
+
 // prune, then F.Add for a successful relaxation of <v2, i> to nd
 template <typename D, int B>
 __device__ __forceinline__ void after_relax(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 f2,
@@ -703,14 +731,10 @@ __device__ __forceinline__ void relax(const EngineArgs& a, GCtx<D>& c, Smem<B>& 
     after_relax<D, B>(a, c, sm, f2, i, v2, pp, nd);
 }
 
-// Process sm.flat[0 .. cnt): extract, update, prune, then relax all edges of
-// the survivors with a load-balanced sweep (consecutive threads read
-// consecutive adjacency entries, 8 bytes each: target and weight).
+// Refresh the prune bounds a CTA of a team reads (no barrier).
 template <typename D, int B>
-__device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 cnt, bool sparse_src,
-                              u32* bm_cur) {
+__device__ __forceinline__ void refresh_bounds(const EngineArgs& a, const GCtx<D>& c, Smem<B>& sm) {
     const u32 t = threadIdx.x;
-    // refresh prune bounds for this tile
     if (t < c.G.scnt) {
         u64 b;
         if (c.G.mode == GM_BIDIR)
@@ -721,6 +745,16 @@ __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 
             b = ldcg64(a.mu + c.G.qbeg);
         sm.bound[t] = b;
     }
+}
+
+// Process sm.flat[0 .. cnt): extract, update, prune, then relax all edges of
+// the survivors with a load-balanced sweep (consecutive threads read
+// consecutive adjacency entries, 8 bytes each: target and weight).
+template <typename D, int B>
+__device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 cnt, bool sparse_src,
+                              u32* bm_cur) {
+    const u32 t = threadIdx.x;
+    refresh_bounds<D, B>(a, c, sm);
     __syncthreads();
     u32 deg = 0;
     u32 xf = 0, xv = 0, xi = 0;  // the survivor this thread extracted (pull-then-push)
@@ -768,11 +802,27 @@ __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 
                     update_bidir<D, B>(a, c, sm, v, i, d);
                 }
                 if (!pruned(pv, sm.bound[i])) {
-                    deg = b1 - b0;
+                    deg = cut_row<D, B>(a, sm, i, d, b0, b1) - b0;
+                    ++c.c_x;
+                    if (a.split && c.slot.ocap && deg > ROW_CHUNK) {
+                        // a long row: in pieces, for the whole team, after
+                        // the tiles (unless the list is full)
+                        const u32 k = (deg + ROW_CHUNK - 1) / ROW_CHUNK;
+                        const u32 at = atomicAdd(&c.S_cur->chunks, k);
+                        const u32 cap = min(c.slot.ocap, c.slot.qcap);
+                        if (at + k <= cap) {
+                            for (u32 j = 0; j < k; ++j) {
+                                c.slot.of[at + j] = f;
+                                reinterpret_cast<u32*>(c.slot.fd[0])[at + j] = b0 + j * ROW_CHUNK;
+                            }
+                            deg = 0;
+                        } else {
+                            for (u32 j = at; j < min(at + k, cap); ++j) c.slot.of[j] = NONE;  // unused places
+                        }
+                    }
                     sm.beg[t] = b0;
                     sm.si[t] = (unsigned char)i;
                     sm.d[t] = d;
-                    ++c.c_x;
                     xf = f;
                     xv = v;
                     xi = i;
@@ -832,6 +882,47 @@ __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 
         relax<D, B>(a, c, sm, sm.si[lo], sm.d[lo], ew, q);
     }
     flush_stage<D, B>(c, sm);
+}
+
+// The second half of a step on graphs with long rows: the team shares the
+// pieces that the tiles put off.  A piece is taken with the row's current
+// distance (at most the one it was put off with).
+template <typename D, int B>
+__device__ void process_chunks(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm) {
+    const u32 t = threadIdx.x;
+    if (t == 0) sm.total = min(ld_volatile(&c.S_cur->chunks), min(c.slot.ocap, c.slot.qcap));
+    refresh_bounds<D, B>(a, c, sm);
+    __syncthreads();
+    const u32 n = sm.total;
+    for (;;) {
+        __syncthreads();
+        if (t == 0) sm.tile = atomicAdd(&c.S_cur->chunk_tile, 1u);
+        __syncthreads();
+        const u32 k = sm.tile;
+        if (k >= n) break;
+        const u32 f = __ldcg(c.slot.of + k);
+        if (f == NONE) continue;
+        const u32 beg = __ldcg(reinterpret_cast<const u32*>(c.slot.fd[0]) + k);
+        u32 v, i;
+        decode_flat(c.G, c.n, f, v, i);
+        const u64 d = ld_dist(c.dist + f);
+        const u32 b1 = min(beg + ROW_CHUNK, __ldg(rows<B>(a, sm, i) + v + 1));
+        const u32 end = cut_row<D, B>(a, sm, i, d, beg, b1);
+        for (u32 e = beg + t; e < end; e += B) {
+            uint2 ew;
+            int2 q = make_int2(0, 0);
+            if (c.adj16) {
+                const int4 r = __ldg(adj16<B>(a, sm, i) + e);
+                ew = make_uint2((u32)r.x, (u32)r.y);
+                q = make_int2(r.z, r.w);
+            } else {
+                ew = __ldg(adj<B>(a, sm, i) + e);
+            }
+            ++c.c_e;
+            relax<D, B>(a, c, sm, i, d, ew, q);
+        }
+        flush_stage<D, B>(c, sm);
+    }
 }
 
 // ----------------------------------------------------------------------------
@@ -1257,7 +1348,7 @@ __device__ void process_local(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, cons
                     update_bidir<D, B>(a, c, sm, v, i, d);
                 }
                 if (!pruned(pv, sm.bound[i])) {
-                    deg = b1 - b0;
+                    deg = cut_row<D, B>(a, sm, i, d, b0, b1) - b0;
                     xb0 = b0;
                     xsi = i;
                     xd = d;
@@ -1833,6 +1924,8 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
             S[0].minkey = 0;
             S[0].tile = 0;
             S[0].overflow = 0;
+            S[0].chunks = S[0].chunk_tile = 0;
+            S[1].chunks = S[1].chunk_tile = 0;
             S[0].cnt_dir[0] = 1;
             S[0].cnt_dir[1] = G.scnt == 2 ? 1 : 0;
             S[0].bmax = INF64;
@@ -1938,12 +2031,14 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
         c.bm_nxt = slot.bm[bnxt];
         c.q_nxt = slot.q[bnxt];
         c.S_nxt = &S[nxt];
+        c.S_cur = &S[cur];
         if (tc.rank == 0 && t == 0) {
             S[old].count = 0;
             S[old].minkey = INF64;
             S[old].tile = 0;
             S[old].overflow = 0;
             S[old].cnt_dir[0] = S[old].cnt_dir[1] = 0;
+            S[old].chunks = S[old].chunk_tile = 0;
             S[old].bmax = INF64;
         }
         if (t == 0) {
@@ -1954,8 +2049,12 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
         ++rounds;
         if (dense_cur) ++dense_rounds;
 
+        // entries of a tile: fewer than B while that leaves CTAs of the team
+        // without one (a step of 8,000 entries on all 152 SMs is 16 tiles of
+        // 512), a warp's worth at least
         if (!dense_cur) {
-            const u32 nt = (count + B - 1) / B;
+            const u32 ts = tc.size == 1 ? (u32)B : min((u32)B, max(32u, count / (2 * tc.size)));
+            const u32 nt = (count + ts - 1) / ts;
             u32 local = tc.rank;
             for (;;) {
                 if (t == 0) sm.tile = tc.size == 1 ? local : atomicAdd(&S[cur].tile, 1u);
@@ -1964,8 +2063,8 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
                 __syncthreads();
                 if (tile >= nt) break;
                 local += tc.size;
-                const u32 base = tile * B;
-                const u32 cnt = min((u32)B, count - base);
+                const u32 base = tile * ts;
+                const u32 cnt = min(ts, count - base);
                 if (t < cnt) sm.flat[t] = __ldcg(slot.q[bcur] + base + t);
                 __syncthreads();
                 process_items<D, B>(a, c, sm, cnt, true, c.bm_cur);
@@ -1999,6 +2098,10 @@ __device__ bool run_group(const EngineArgs& a, const TeamCtx& tc, const SlotDev&
                     process_items<D, B>(a, c, sm, min((u32)B, total - base), false, c.bm_cur);
                 }
             }
+        }
+        if (a.split && slot.ocap) {
+            if (!team_sync(tc, a, &sm.flag)) return false;
+            process_chunks<D, B>(a, c, sm);
         }
         // flush per-CTA step results
         __syncthreads();

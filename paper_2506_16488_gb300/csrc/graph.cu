@@ -221,6 +221,10 @@ static bool locality_order(u64 n, const float* xy, std::vector<u32>& perm, std::
     return true;
 }
 
+// Largest average degree of a graph with adjacency blocks (road and grid
+// shapes have 3.6 to 4, so most rows fit a block of four).
+constexpr u64 BLOCK_MAX_DEG = 6;
+
 SlotCaps slot_caps(u64 range, int frontier, bool whole_gpu) {
     u64 fc = std::max<u64>(range, 64);
     fc = (fc + 63) & ~63ull;
@@ -425,6 +429,19 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         weights = w_r.data();
         coords = xy_r.data();
     }
+    // Rows sorted by weight where rows are long (graphs without adjacency
+    // blocks): a search that has a bound on its answer stops scanning a row at
+    // the first edge that reaches it (cut_row in engine_core.cuh).  Nothing else
+    // depends on the order within a row.
+    g->wsorted = m > BLOCK_MAX_DEG * n;
+    auto sort_rows = [](u64 rows, const auto* off, uint2* ed) {
+        parallel_for(rows, [&](u64 lo, u64 hi, unsigned) {
+            for (u64 v = lo; v < hi; ++v)
+                std::sort(ed + off[v], ed + off[v + 1], [](const uint2& x, const uint2& y) {
+                    return x.y != y.y ? x.y < y.y : x.x < y.x;
+                });
+        });
+    };
     ppsp_graph_info& info = g->info;
     info.n = n;
     info.m = m;
@@ -460,6 +477,7 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
     for (u64 v = 0; v <= n; ++v) off32[v] = (u32)offsets[v];
     std::vector<uint2> ed(m);
     for (u64 e = 0; e < m; ++e) ed[e] = make_uint2(targets[e], weights[e]);
+    if (g->wsorted) sort_rows(n, offsets, ed.data());
     cudaError_t ce;
     if ((ce = cudaGetDevice(&g->device)) != cudaSuccess) {
         set_last_cuda_error(ce, "cudaGetDevice", __FILE__, __LINE__);
@@ -509,6 +527,7 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         edt.resize(m);
         for (u64 u = 0; u < n; ++u)
             for (u64 e = offsets[u]; e < offsets[u + 1]; ++e) edt[fill[targets[e]]++] = make_uint2((u32)u, weights[e]);
+        if (g->wsorted) sort_rows(n, offt.data(), edt.data());
         if ((ce = cudaMalloc(&g->d_off_t, (n + 1) * 4)) != cudaSuccess) return fail(ce, "cudaMalloc(off_t)");
         if ((ce = cudaMalloc(&g->d_edges_t, std::max<u64>(1, m) * 8)) != cudaSuccess)
             return fail(ce, "cudaMalloc(edges_t)");
@@ -542,7 +561,7 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
                              scaled ? (int)g->pc_host[2 * (u64)v + 1] : 0);
         };
         std::vector<int4> e16(std::max<u64>(1, m));
-        for (u64 e = 0; e < m; ++e) e16[e] = rec(targets[e], weights[e]);
+        for (u64 e = 0; e < m; ++e) e16[e] = rec(ed[e].x, ed[e].y);
         if ((ce = cudaMalloc(&g->d_edges_pc, std::max<u64>(1, m) * 16)) != cudaSuccess)
             return fail(ce, "cudaMalloc(edges_pc)");
         if (m && (ce = cudaMemcpy(g->d_edges_pc, e16.data(), m * 16, cudaMemcpyHostToDevice)) != cudaSuccess)
@@ -558,10 +577,8 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         }
     }
     // Adjacency blocks for the bucketed kernel: graphs of average degree at
-    // most BLOCK_MAX_DEG (road and grid shapes have 3.6 to 4).  They are left
-    // out, and plans run over the offsets, when they would take more than an
+    // most BLOCK_MAX_DEG.  They are left out, and plans run over the offsets, when they would take more than an
     // eighth of the free device memory or a record index 32 bits.
-    constexpr u64 BLOCK_MAX_DEG = 6;
     if (m <= BLOCK_MAX_DEG * n && n < (1ull << 29)) {
         const u32 dirs = info.undirected ? 1 : 2;
         std::vector<u32> more[2];  // record index of the continued edges, per direction

@@ -46,6 +46,7 @@ struct ppsp_graph {
     ppsp::u32* d_off_t = nullptr;  // transpose of a directed graph (null when undirected)
     uint2* d_edges_t = nullptr;
     int2* d_pc = nullptr;
+    bool wsorted = false;          // rows sorted by weight on the device
     uint64_t device_mem = 0;       // total memory of the device
     void* d_blocks = nullptr;      // adjacency blocks (GraphDev::blk8 ...), one allocation, or null
     uint2* d_blk8 = nullptr;
@@ -86,7 +87,7 @@ struct ppsp_graph {
         g.n = (ppsp::u32)n;
         g.pot_shift = (ppsp::u32)pot_shift;
         g.m = (ppsp::u32)m;
-        g.pad = 0;
+        g.wsorted = wsorted ? 1u : 0u;
         return g;
     }
 };

@@ -136,6 +136,7 @@ __global__ void na_setup_kernel(unsigned char* base, u32 s, u32 t, u64 m, u64 de
     sd->q[1] = reinterpret_cast<u32*>(base + O_Q1);
     sd->touched = reinterpret_cast<u32*>(base + O_TOUCH);
     sd->memo = nullptr;
+    sd->ocap = 0;  // no overflow lists: long rows are not split
     sd->st = reinterpret_cast<SlotState*>(base + O_SLOTST);
     sd->flat_cap = NA_FLAT;
     sd->qcap = NA_QCAP;

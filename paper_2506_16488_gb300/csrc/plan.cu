@@ -708,7 +708,10 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     if (o.delta == 0 && g->delta_model[o.mode] != nullptr) P->model = g->delta_model[o.mode];
 
     // ---- launch shape ----
-    int block = o.block_threads ? o.block_threads : 512;
+    // teams of several CTAs: 512 threads (128 registers), or 1,024 (64) where
+    // rows are long and the edge loop, which needs few registers, dominates
+    // (RMAT-20: 75 groups 174 against 130 ms on teams of eight)
+    int block = o.block_threads ? o.block_threads : (g->wsorted ? 1024 : 512);
     int bpsm = 0, sms = 0;
     u32 ring_cap = o.ring_entries ? o.ring_entries : RING_CAP_DEFAULT;
     st = engine_occupancy(o.dist_bits, block, &bpsm, &sms, ENGINE_GENERAL, ring_cap);
@@ -720,7 +723,11 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
 
     // ---- teams and queues ----
     std::vector<u32> big, small;
-    for (u32 gi = 0; gi < NG; ++gi) (P->groups[gi].scnt > 2 ? big : small).push_back(gi);
+    bool any_sssp = false;
+    for (u32 gi = 0; gi < NG; ++gi) {
+        (P->groups[gi].scnt > 2 ? big : small).push_back(gi);
+        any_sssp = any_sssp || P->groups[gi].mode == GM_SSSP;
+    }
     auto by_work = [&](u32 a, u32 b) { return gwork[a] > gwork[b]; };
     std::stable_sort(big.begin(), big.end(), by_work);
     std::stable_sort(small.begin(), small.end(), by_work);
@@ -760,6 +767,17 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 // fewer groups than CTAs: give each group a team of several CTAs
                 u32 ts_auto = 1;
                 while (ts_auto * 2 <= 32 && (u64)ts_auto * 2 * small.size() <= g_small) ts_auto *= 2;
+                // Graphs with long rows (RMAT shapes): eight CTAs at least,
+                // which take the groups in turn, longest first: a group's
+                // steps are large enough to share, and the longest one (a
+                // search with many targets) no longer outlasts the rest.
+                // RMAT-20, teams of 2 / 4 / 8 / 16: 75 single-source groups
+                // 225 / 160 / 130 / 195 ms, 24 of them 172 / 88 / 51 / 56, 300
+                // 468 / 377 / 375 / 576 (one CTA each: 2,490), 24 pairs 199 /
+                // 98 / 54 / 34.  More pairs than CTAs stay on one CTA each
+                // (300: 205 against 231).
+                if (g->wsorted && (any_sssp || small.size() <= g_small))
+                    ts_auto = std::max<u32>(ts_auto, std::min<u32>(8, g_small));
                 u32 ts = o.team_ctas ? std::min<u32>((u32)o.team_ctas, g_small) : ts_auto;
                 // no more teams than groups: an idle team would still hold a slot
                 u32 nst = std::max<u32>(1, std::min<u32>(g_small / ts, (u32)small.size()));
@@ -1014,6 +1032,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     a.memo = P->memo ? 1u : 0u;
     a.ring_cap = ring_cap;
     a.pull = (o.pull_push && g->info.undirected) ? 1u : 0u;
+    a.split = (!a.pull && g->info.deg_max > ROW_CHUNK) ? 1u : 0u;
     a.debug = o.debug_flags;
     a.spin_limit = o.spin_limit ? o.spin_limit : (1ull << 26);
     a.err = (u32*)(base + o_err);

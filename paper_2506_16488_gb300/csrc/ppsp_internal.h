@@ -25,6 +25,11 @@ typedef int64_t i64;
 constexpr u64 INF64 = ~0ull;
 constexpr u32 INF32 = ~0u;
 constexpr u32 NONE = ~0u;
+// Edges of one piece of a row that a team shares (queue / bitmap path).  A row
+// of RMAT-20 has up to 60,000 edges, which one CTA scanned alone while the
+// others waited: one query 17.8 -> 4.2 ms together with smaller tiles and rows
+// cut at the bound (cut_row).
+constexpr u32 ROW_CHUNK = 2048;
 constexpr int KMAX = 64;          // searches per group (query-graph vertices)
 constexpr int MAX_QUEUES = 2;     // group queues: 0 = multi-search groups, 1 = pairs/singles
 
@@ -71,7 +76,7 @@ struct GraphDev {
     u32 n;
     u32 pot_shift;        // F: h = isqrt(d2 >> 2F)
     u32 m;                // adjacency entries (bounds of checked builds)
-    u32 pad;
+    u32 wsorted;          // rows are sorted by weight
 };
 
 struct SearchDev {
@@ -111,6 +116,8 @@ struct StepState {
     u32 tile;             // dynamic tile counter while the step is processed
     u32 overflow;         // queue overflowed: step must be processed from the bitmap
     u32 cnt_dir[2];       // entries per direction (two-search groups)
+    u32 chunks;           // pieces of long rows put off to the step's second half
+    u32 chunk_tile;       // the next piece to take
     u32 pad;
     u64 bmax;             // largest prune bound of the group, taken before the step's barrier
 };
@@ -172,6 +179,7 @@ struct EngineArgs {
     u32 frontier;         // PPSP_FRONTIER_*
     u32 rho;              // one-CTA path: a step takes buckets until it holds >= rho entries (0 = one)
     u32 memo;             // memoize potential terms in the slot (Sec. 5)
+    u32 split;            // queue / bitmap path: rows longer than ROW_CHUNK are shared by the team
     u32 pull;             // queue / bitmap path: pull before push (App. B), undirected graphs
     u32 ring_cap;         // one-CTA path: shared-memory entries per bucket (1 .. 256)
     u32 debug;
