@@ -111,7 +111,8 @@ typedef struct {
     int32_t mode;            /* PPSP_BIDS (default) ... PPSP_ASTAR                         */
     int32_t dist_bits;       /* 32 (default) or 64: width of tentative distances in HBM     */
     uint64_t delta;          /* stepping increment Delta >= 1; 0 = auto (learned model if
-                                attached to the graph, else mean edge weight)               */
+                                attached to the graph, else mean edge weight, a sixth to a
+                                32nd of it by the query's distance with A* potentials)      */
     int32_t frontier;        /* PPSP_FRONTIER_* (default AUTO)                              */
     int32_t layout;          /* PPSP_LAYOUT_* (default AUTO)                                */
     int32_t batch_strategy;  /* PPSP_BATCH_* (default MULTI)                                */

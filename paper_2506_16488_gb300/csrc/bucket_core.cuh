@@ -1,6 +1,7 @@
 // Bucketed search kernel for graphs of low degree (road and grid shapes): one
-// CTA runs a group of one or two searches to completion, and a team of CTAs a
-// Multi-BiDS group, one search each (see bk_update).
+// CTA, or a cluster of them (see bk_gather), runs a group of one or two
+// searches to completion, and a team of CTAs a Multi-BiDS group, one search
+// each (see bk_update).
 //
 // Same algorithm as run_local (engine_core.cuh): Delta*-stepping buckets in
 // shared memory with lazy deletion, a far list beyond the ring's window, a
@@ -61,6 +62,18 @@ constexpr u32 BK_EXTRA = 1u << 31;  // of a ring entry: the vertex's continued e
 enum { BK_BIDS = 0, BK_BIDASTAR = 1, BK_SINGLE = 2, BK_MULTI = 3 };
 constexpr bool bk_one(int kind) { return kind == BK_SINGLE || kind == BK_MULTI; }
 
+// How a group of one or two searches is run, and the kernel's instances: by
+// one CTA; the same, with teams of CTAs for the larger groups; by a cluster.
+enum { BK_CTAS = 0, BK_TEAMS = 1, BK_CLUSTERS = 2 };
+constexpr u32 BK_CL_MAX = 8;  // CTAs of a cluster (the portable limit)
+
+// What the CTAs of a cluster tell each other at the end of a step.
+struct BkPub {
+    u64 far_min, bound;
+    u32 far_n, full, late, spill, fresh, cnt0, cnt1, pad;
+    u32 rn[BK_NB];
+};
+
 struct BkShared {
     // the decision of a step, read by every thread
     u64 cur, curkey;      // the bucket of the step and its threshold cur * step
@@ -82,6 +95,10 @@ struct BkShared {
     u32 src[2], sdir[2], pcnt[2];
     PartnerDev pcache[2];
     u32 group, flag;
+    // clusters: published states (two in turn), and the entries that CTAs 0 ..
+    // r - 1 hold of the step's bucket; this CTA takes entries e0 .. n - 1 of all
+    BkPub pub[2];
+    u32 pre[BK_CL_MAX + 1], e0, any_spill;
     // a Multi-BiDS search: its partners j, their query edges and mu (mirrors,
     // never below a.mu); muj[j] = 0 where j is no partner
     u32 pj[KMAX], npart;
@@ -122,6 +139,7 @@ struct BkCtx {
     u32 tcap;
     u32 mode, target, qe;
     u32 d0, dm;   // direction of search i: d0 | (i & dm)
+    u32 cl, rank; // cluster: its CTAs and this one's place
     u32 ks, i0;   // one search of a group: its distances are dist[(v << ks) | i0]
     u32 magic;    // floor(2^32 / step)
     u32 cur_lo;   // this step's bucket (low bits)
@@ -421,21 +439,31 @@ __device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkSha
 }
 
 // Take the bucket's entries: four lanes each.
-template <typename D, int B, int KIND>
+template <typename D, int B, int KIND, bool CL>
 __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot) {
     constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
     const u32 t = threadIdx.x, q4 = t & 3u;
     const u32 n = sm.n, s = sm.slot;
-    for (u32 e = t >> 2; e < n; e += B / 4) {
-        u32 f;
+    for (u32 e1 = (CL ? sm.e0 : 0u) + (t >> 2); e1 < n; e1 += B / 4) {
+        u32 f, e = e1;
         u64 dins;
+        const typename BkEntry<D>::T* ring = c.ring;
+        i64 ovf = (i64)((size_t)s * c.ob);
+        if (CL) {
+            // the entry's holder: its shared memory and its overflow region
+            u32 r = 0;
+            while (e1 >= sm.pre[r + 1]) ++r;
+            e = e1 - sm.pre[r];
+            ring = cg::this_cluster().map_shared_rank(c.ring, r);
+            ovf += ((i64)r - (i64)c.rank) * (i64)sm.dev.ocap;
+        }
         if (e < c.cap) {
-            const typename BkEntry<D>::T x = c.ring[s * c.cap + e];
+            const typename BkEntry<D>::T x = ring[s * c.cap + e];
             f = (u32)x.x;
             dins = x.y;
         } else {
-            f = __ldcg(sm.dev.of + (size_t)s * c.ob + (e - c.cap));
-            dins = ld_dist(reinterpret_cast<const D*>(sm.dev.od) + (size_t)s * c.ob + (e - c.cap));
+            f = __ldcg(sm.dev.of + ovf + (e - c.cap));
+            dins = ld_dist(reinterpret_cast<const D*>(sm.dev.od) + ovf + (e - c.cap));
         }
         const u32 extra = f & BK_EXTRA;
         f &= ~BK_EXTRA;
@@ -562,7 +590,7 @@ template <typename D, int B, int KIND>
 __device__ __forceinline__ void bk_recover(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, bool pot, u32 nwords) {
     if (threadIdx.x == 0) sm.spill = 0;
     __syncthreads();
-    for (u32 w = threadIdx.x; w < nwords; w += B) {
+    for (u32 w = c.rank * B + threadIdx.x; w < nwords; w += c.cl * B) {
         u32 bits = __ldcg(sm.dev.bm[0] + w);
         if (!bits) continue;
         // cleared before its entries are inserted again: one that spills once
@@ -576,16 +604,102 @@ __device__ __forceinline__ void bk_recover(const EngineArgs& a, BkCtx<D>& c, BkS
     }
 }
 
+// A cluster runs one group: relaxed entries go to the ring of the CTA that
+// relaxed them, and a step takes the bucket's entries of all rings, split
+// evenly (read through distributed shared memory).  Each CTA publishes its
+// state at the end of a step, the cluster meets at one hardware barrier, and
+// every CTA makes the same decision from all states.  A step gains a barrier
+// (400-600 cycles) and the reads of the others' states (225 each way), 2 us in
+// all, so clusters are for steps of more entries than one CTA takes in a pass
+// or two (bucket_group_us in plan.cu).  Measured, one CTA / eight, six queries
+// one after the other: BiDS on the 2048^2 road graph 108 / 52 ms, ET 228 / 81
+// (the queue / bitmap frontier on all CTAs: 105, 96), BiD-A* on 1024^2 11 / 16;
+// a 64-leaf star on 2048^2 104 / 25 ms (46 on 32 CTAs of the queue path);
+// 256 BiD-A* queries with 64-bit distances on 4096^2, clusters of two: 136 ->
+// 106 ms, because the longest queries outlast the rest.
+__device__ __forceinline__ void bk_publish(BkShared& sm, u32 par, bool fresh) {
+    const u32 t = threadIdx.x;
+    BkPub& p = sm.pub[par];
+    p.rn[t] = sm.rn[t];
+    p.rn[t + 32] = sm.rn[t + 32];
+    if (t == 0) {
+        p.far_n = sm.far_n;
+        p.far_min = sm.far_min;
+        p.full = sm.far_n > sm.dev.qcap / 2 && sm.far_n > 2 * sm.far_after;
+        p.bound = sm.bound;
+        p.late = sm.late;
+        p.spill = sm.spill;
+        p.fresh = fresh;
+        p.cnt0 = sm.cnt_dir[0];
+        p.cnt1 = sm.cnt_dir[1];
+    }
+}
+
+// The state a decision is made from: one CTA's, or all of a cluster's.
+struct BkState {
+    u32 n0, n1;           // entries of buckets cur + 1 + lane and cur + 33 + lane
+    u64 bound, far_min;
+    u32 late, spill, farn, full, dry;
+};
+
+__device__ __forceinline__ u64 bk_min64(u64 x) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        const u64 y = __shfl_xor_sync(0xffffffffu, x, o);
+        x = y < x ? y : x;
+    }
+    return __shfl_sync(0xffffffffu, x, 0);
+}
+
+__device__ __forceinline__ BkState bk_gather(BkShared& sm, u32 cl, u32 par, u32 lo) {
+    const u32 t = threadIdx.x;
+    cg::cluster_group g = cg::this_cluster();
+    BkState s;
+    s.n0 = s.n1 = 0;
+    for (u32 r = 0; r < cl; ++r) {
+        const BkPub* p = g.map_shared_rank(&sm.pub[par], r);
+        s.n0 += p->rn[(lo + 1 + t) & (BK_NB - 1)];
+        if (t < 31) s.n1 += p->rn[(lo + 33 + t) & (BK_NB - 1)];
+    }
+    const bool on = t < cl;  // lane r < cl reads CTA r's scalars (cl <= 8: reduced over 8 lanes)
+    const BkPub* p = g.map_shared_rank(&sm.pub[par], on ? t : 0u);
+    const u32 far = on ? p->far_n : 0u;
+    s.bound = bk_min64(on ? p->bound : INF64);
+    s.far_min = bk_min64(far ? p->far_min : INF64);
+    s.farn = __reduce_add_sync(0xffffffffu, far ? 1u : 0u);
+    s.late = __reduce_max_sync(0xffffffffu, on ? p->late : 0u);
+    s.spill = __reduce_or_sync(0xffffffffu, on ? p->spill : 0u);
+    s.full = __reduce_or_sync(0xffffffffu, on ? p->full : 0u);
+    const u32 c0 = __reduce_add_sync(0xffffffffu, on ? p->cnt0 : 0u);
+    const u32 c1 = __reduce_add_sync(0xffffffffu, on ? p->cnt1 : 0u);
+    s.dry = __all_sync(0xffffffffu, !on || p->fresh) && (c0 == 0 || c1 == 0);
+    return s;
+}
+
 // The next step, decided by the first warp (every lane computes the same).
 // fresh: the entry counts per direction are up to date.
-template <typename D, int KIND>
-__device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c, BkShared& sm, bool fresh) {
+template <typename D, int KIND, bool CL>
+__device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c, BkShared& sm, bool fresh, u32 par) {
     const u32 t = threadIdx.x;
-    const u64 cur = sm.cur, curkey = sm.curkey, bound = sm.bound, step = sm.step, fmin = sm.far_min;
+    const u64 cur = sm.cur, curkey = sm.curkey, step = sm.step;
     const i64 koff = sm.key_off;
-    const u32 lo = (u32)cur, spill = sm.spill, late = sm.late, farn = sm.far_n;
-    const u32 n0 = sm.rn[(lo + 1 + t) & (BK_NB - 1)];
-    const u32 n1 = t < 31 ? sm.rn[(lo + 33 + t) & (BK_NB - 1)] : 0u;
+    const u32 lo = (u32)cur;
+    BkState st;
+    if (CL) {
+        st = bk_gather(sm, c.cl, par, lo);
+    } else {
+        st.n0 = sm.rn[(lo + 1 + t) & (BK_NB - 1)];
+        st.n1 = t < 31 ? sm.rn[(lo + 33 + t) & (BK_NB - 1)] : 0u;
+        st.bound = sm.bound;
+        st.far_min = sm.far_min;
+        st.late = sm.late;
+        st.spill = sm.spill;
+        st.farn = sm.far_n;
+        st.full = st.farn > sm.dev.qcap / 2 && st.farn > 2 * sm.far_after;
+        st.dry = fresh && (sm.cnt_dir[0] == 0 || sm.cnt_dir[1] == 0);
+    }
+    const u64 bound = st.bound, fmin = st.far_min;
+    const u32 n0 = st.n0, n1 = st.n1, spill = st.spill, late = st.late, farn = st.farn;
     const u32 m0 = __ballot_sync(0xffffffffu, n0 != 0), m1 = __ballot_sync(0xffffffffu, n1 != 0);
     // buckets ahead of the current one: first non-empty one of the ring, and
     // of the far list (FAR: none, or at least that many)
@@ -604,18 +718,18 @@ __device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c
         if (kn == 1 && late) ahead = late != 0xFFFFFFFFu ? 1 - (i64)late : -(i64)curkey;
         stop = !spill && bound > 0 && (i64)curkey + ahead - koff >= (i64)bound;
     } else {
-        stop = !bk_one(KIND) && fresh && (sm.cnt_dir[0] == 0 || sm.cnt_dir[1] == 0);
+        stop = !bk_one(KIND) && st.dry;
     }
     u32 what = 0, ahead = k;
     if (stop) {
         what = 3;
-    } else if (spill || k == FAR || (farn && (kf <= k || kf < BK_NB / 2 || farn > sm.dev.qcap / 2))) {
+    } else if (spill || k == FAR || (farn && (kf <= k || kf < BK_NB / 2 || st.full))) {
         const bool none = k == FAR && !farn;
         if (spill && (!sm.recov || none)) {
             // recover spilled entries before they fall behind, at most once
             // between two processed buckets
             what = 2;
-        } else if (farn && (kf <= k || kf < BK_NB / 2 || (farn > sm.dev.qcap / 2 && farn > 2 * sm.far_after))) {
+        } else if (farn && (kf <= k || kf < BK_NB / 2 || st.full)) {
             // far entries due soon, an empty ring, or a far list filling up
             // with stale entries (re-bucketing drops them)
             what = 1;
@@ -623,9 +737,31 @@ __device__ __forceinline__ void bk_decide(const EngineArgs& a, const BkCtx<D>& c
             what = spill ? 2 : 3;
         }
     }
+    if (CL && what == 0) {
+        // the bucket's entries per CTA, and this one's share of them
+        u32 x = 0;
+        if (t < c.cl)
+            x = min(cg::this_cluster().map_shared_rank(&sm.pub[par], t)->rn[(lo + k) & (BK_NB - 1)], c.cap + c.ob);
+#pragma unroll
+        for (int o = 1; o < (int)BK_CL_MAX; o <<= 1) {
+            const u32 y = __shfl_up_sync(0xffffffffu, x, o);
+            if (t >= (u32)o) x += y;
+        }
+        const u32 total = __shfl_sync(0xffffffffu, x, c.cl - 1), share = (total + c.cl - 1) / c.cl;
+        if (t < c.cl) sm.pre[t + 1] = x;
+        if (t == 0) {
+            sm.pre[0] = 0;
+            sm.e0 = min(c.rank * share, total);
+            sm.n = min(c.rank * share + share, total);
+        }
+    }
     if (t == 0) {
+        if (CL) {
+            sm.bound = bound;
+            sm.any_spill = spill;
+        }
         if (what == 0) {
-            sm.n = min(nn, c.cap + c.ob);
+            if (!CL) sm.n = min(nn, c.cap + c.ob);
             sm.slot = (lo + k) & (BK_NB - 1);
             sm.recov = 0;
             sm.idle = 0;
@@ -689,11 +825,11 @@ __device__ __forceinline__ void bk_flush_dir(BkCtx<D>& c, BkShared& sm) {
 
 // One group, or (BK_MULTI) search `rank` of one.  Returns false when a wait of
 // the team ran out.
-template <typename D, int B, int KIND>
+template <typename D, int B, int KIND, bool CL>
 __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc, u32 gi, const GroupDev& G,
                                          BkShared& sm, unsigned char* ring) {
     constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
-    const u32 t = threadIdx.x, rank = KIND == BK_MULTI ? tc.rank : 0u;
+    const u32 t = threadIdx.x, rank = KIND == BK_MULTI || CL ? tc.rank : 0u;
     const u64 t_start = (a.group_ns && t == 0 && rank == 0) ? global_ns() : 0;
     BkCtx<D> c;
     c.dist = reinterpret_cast<D*>(sm.dev.dist);
@@ -707,14 +843,17 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
     c.qe = G.qbeg;
     c.ks = KIND == BK_MULTI ? G.kshift : 0u;
     c.i0 = rank;
+    c.cl = CL ? tc.size : 1u;
+    c.rank = CL ? rank : 0u;
     c.c_x = c.c_e = c.c_r = c.c_p = c.c_t = 0;
     c.dc0 = c.dc1 = 0;
     const u32 flat_range = a.g.n << KS, nwords = (flat_range + 31u) >> 5;
     const u64 step = KIND != BK_SINGLE ? 2 * G.delta : G.delta;
     const u32 scnt = KIND == BK_MULTI ? 1u : G.scnt;  // searches of this CTA
     u32 sdeg = 0;
+    const bool lead = !CL || rank == 0;  // a cluster's first CTA starts the searches
     if (t < scnt) {
-        const SearchDev s = a.searches[G.sbeg + rank + t];
+        const SearchDev s = a.searches[G.sbeg + (KIND == BK_MULTI ? rank : 0u) + t];
         const u32* off = s.dir ? a.g.off_t : a.g.off;
         sdeg = __ldg(off + s.src + 1) - __ldg(off + s.src);
         sm.src[t] = s.src;
@@ -722,8 +861,10 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
         sm.pcnt[t] = s.pcnt;
         if (KIND != BK_MULTI && s.pcnt) sm.pcache[t] = a.partners[s.pbeg];
         const u32 f = (s.src << KS) | t;
-        st_dist(bk_at<D, KIND>(c, f), 0);
-        c.touched[t] = f;
+        if (lead) {
+            st_dist(bk_at<D, KIND>(c, f), 0);
+            c.touched[t] = f;
+        }
         if (t == 0) {
             sm.key_off = KIND == BK_MULTI ? 0 : s.key_off;
             sm.npart = s.pcnt;
@@ -742,7 +883,7 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
         sm.late = 0;
         sm.far_n = sm.far_at = sm.far_after = 0;
         sm.far_min = INF64;
-        sm.tn = scnt;
+        sm.tn = lead ? scnt : 0u;
         sm.tov = sm.spill = sm.recov = sm.idle = sm.ndef = 0;
         sm.cnt_dir[0] = sm.cnt_dir[1] = 0;
     }
@@ -767,13 +908,17 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
     c.cur_lo = 0;
     c.kc = sm.key_off;
     // Init: the sources (key 0) go to the first step
-    if (t < scnt) bk_insert<D, KIND>(c, sm, (sm.src[t] << KS) | t, sdeg > 4 ? 2u : 0u, -sm.key_off, 0);
+    if (lead && t < scnt) bk_insert<D, KIND>(c, sm, (sm.src[t] << KS) | t, sdeg > 4 ? 2u : 0u, -sm.key_off, 0);
     bk_flush_dir<D, KIND>(c, sm);
     __syncthreads();
     u64 rounds = 0;
     bool fresh = false;
-    for (;;) {
-        if (t < 32) bk_decide<D, KIND>(a, c, sm, fresh);
+    for (u32 par = 0;; par ^= 1u) {
+        if (CL) {
+            if (t < 32) bk_publish(sm, par, fresh);
+            cg::this_cluster().sync();
+        }
+        if (t < 32) bk_decide<D, KIND, CL>(a, c, sm, fresh, par);
         __syncthreads();
         const u32 what = sm.what;
         if (what == 3) break;
@@ -781,8 +926,8 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
         c.kc = sm.key_off - (i64)sm.curkey;
         fresh = false;
         if (what == 0) {
-            bk_process<D, B, KIND>(a, c, sm, pot);
-            if (KIND == BK_SINGLE && c.mode == GM_SSSP && t >= B - 32 && (rounds & 3) == 0) {
+            bk_process<D, B, KIND, CL>(a, c, sm, pot);
+            if (KIND == BK_SINGLE && c.mode == GM_SSSP && lead && t >= B - 32 && (rounds & 3) == 0) {
                 __syncwarp();
                 const u64 m = bk_target_max<D>(a, c, G);
                 if (t == B - 32) atomicMin(reinterpret_cast<unsigned long long*>(&sm.bound), (unsigned long long)m);
@@ -813,9 +958,10 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
         }
     }
     // entries left in the spill bitmap by an early stop
-    if (sm.spill)
-        for (u32 w = t; w < nwords; w += B) sm.dev.bm[0][w] = 0u;
-    if (KIND == BK_SINGLE && c.mode == GM_SSSP) {
+    if (CL) cg::this_cluster().sync();  // every CTA has made the last decision, and its writes are done
+    if (CL ? sm.any_spill : sm.spill)
+        for (u32 w = c.rank * B + t; w < nwords; w += c.cl * B) sm.dev.bm[0][w] = 0u;
+    if (KIND == BK_SINGLE && c.mode == GM_SSSP && lead) {
         for (u32 q = t; q < G.qcnt; q += B) {
             const u64 d = ld_dist(c.dist + a.qedges[G.qbeg + q].b);
             a.mu[G.qbeg + q] = (d == DT<D>::INF) ? INF64 : d;
@@ -823,7 +969,7 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
     }
     const u32 tn = min(sm.tn, c.tcap);
     const bool tov = sm.tov != 0;
-    if (KIND != BK_MULTI && a.path_buf != nullptr) {
+    if (KIND != BK_MULTI && !CL && a.path_buf != nullptr) {
         __syncthreads();
         TeamCtx one{0, 0, 1, nullptr, false, 1};
         GCtx<D> g;
@@ -836,6 +982,8 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
     if (KIND == BK_MULTI) {
         // the other searches read these distances until they end, too
         if (!team_sync(tc, a, &sm.flag)) return false;
+    } else if (CL) {
+        cg::this_cluster().sync();  // the answers are read
     } else {
         __syncthreads();
     }
@@ -856,7 +1004,7 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
             for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
             if ((t & 31u) == 0 && x) atomicAdd(cp + at[k], (unsigned long long)x);
         }
-        if (t == 0) {
+        if (t == 0 && lead) {
             atomicAdd(cp + 4, (unsigned long long)rounds);
             if (rank == 0) atomicAdd(cp + 5, 1ull);
             atomicAdd(cp + 6, (unsigned long long)scnt);
@@ -873,29 +1021,31 @@ struct BucketMinBlocks {
     static constexpr int value = 1024 / B;
 };
 
-// TEAMS = false: each CTA is a team that takes groups from its queue; no CTA
-// waits for another one, so the launch is an ordinary one.  TEAMS: some teams
+// BK_CTAS: each CTA is a team that takes groups from its queue; no CTA waits
+// for another one, so the launch is an ordinary one.  BK_TEAMS: some teams
 // have several CTAs and run Multi-BiDS groups, one search per CTA (a
 // cooperative launch: the CTAs of a team meet when a group starts and ends).
-template <typename D, int B, bool TEAMS>
+// BK_CLUSTERS: each cluster of a.cluster CTAs is a team.
+template <typename D, int B, int RUN>
 __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(EngineArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BkShared& sm = *reinterpret_cast<BkShared*>(smem_raw);
     unsigned char* ring = smem_raw + ((sizeof(BkShared) + 15) & ~(size_t)15);
     TeamCtx tc;
-    tc.team = TEAMS ? a.cta_team[blockIdx.x] : blockIdx.x;
-    tc.rank = TEAMS ? blockIdx.x - a.team_first[tc.team] : 0u;
-    tc.size = TEAMS ? a.team_size[tc.team] : 1u;
+    tc.team = RUN == BK_TEAMS ? a.cta_team[blockIdx.x] : RUN == BK_CLUSTERS ? blockIdx.x / a.cluster : blockIdx.x;
+    tc.rank = RUN == BK_TEAMS ? blockIdx.x - a.team_first[tc.team] : RUN == BK_CLUSTERS ? blockIdx.x % a.cluster : 0u;
+    tc.size = RUN == BK_TEAMS ? a.team_size[tc.team] : RUN == BK_CLUSTERS ? a.cluster : 1u;
     tc.ts = a.tstate + tc.team;
-    tc.global_bar = tc.size > 1;
+    tc.global_bar = RUN == BK_TEAMS && tc.size > 1;
     tc.expect = tc.size;
     tc.wait_shift = 4;
     const u32 qid = a.team_queue[tc.team];
     if (threadIdx.x == 0) {
         SlotDev s = a.slots[tc.team];
-        if (TEAMS && tc.size > 1) {
-            // this CTA's share of the slot's lists; its spill bitmap covers
-            // the vertices, and both bitmaps together hold one per search
+        if (RUN != BK_CTAS && tc.size > 1) {
+            // this CTA's share of the slot's lists.  The spill bitmap is
+            // shared by a cluster; a search of a team has its own over the
+            // vertices, of which both bitmaps together hold one per search
             // (n bits each, rounded up to words, of 2n per search)
             const u32 r = tc.rank, k = tc.size;
             s.ocap = s.ocap / k / BK_NB * BK_NB;
@@ -908,101 +1058,154 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
                 s.fd[x] = reinterpret_cast<D*>(s.fd[x]) + (size_t)r * s.qcap;
             }
             s.touched += (size_t)r * s.tcap;
-            s.bm[0] += (size_t)r * ((a.g.n + 31u) / 32u);
+            if (RUN == BK_TEAMS) s.bm[0] += (size_t)r * ((a.g.n + 31u) / 32u);
         }
         sm.dev = s;
     }
+    if (RUN == BK_CLUSTERS) cg::this_cluster().sync();  // every CTA runs before its shared memory is written
     for (;;) {
         if (threadIdx.x == 0 && tc.rank == 0) {
             const u32 idx = atomicAdd(a.queue_head + qid, 1u);
             const u32 g = idx < a.queue_len[qid] ? a.queue_items[qid][idx] : NONE;
-            if (TEAMS && tc.global_bar) tc.ts->group = g;
-            sm.group = g;
+            if (tc.global_bar) tc.ts->group = g;
+            if (RUN == BK_CLUSTERS)
+                for (u32 r = 0; r < tc.size; ++r) *cg::this_cluster().map_shared_rank(&sm.group, r) = g;
+            else
+                sm.group = g;
         }
-        if (TEAMS && tc.global_bar) {
+        if (RUN == BK_TEAMS && tc.global_bar) {
             if (!team_sync(tc, a, &sm.flag)) break;
             if (threadIdx.x == 0) sm.group = ld_volatile(&tc.ts->group);
         }
-        __syncthreads();
+        if (RUN == BK_CLUSTERS)
+            cg::this_cluster().sync();
+        else
+            __syncthreads();
         const u32 gi = sm.group;
         if (gi == NONE) break;
         const GroupDev G = a.groups[gi];
-        if (TEAMS && tc.global_bar) {
+        if (RUN == BK_TEAMS && tc.global_bar) {
             // the team meets when the group starts, when its searches end
             // and (above) before the next one is claimed
             if (tc.rank < G.scnt) {
-                if (!bk_group<D, B, BK_MULTI>(a, tc, gi, G, sm, ring)) break;
+                if (!bk_group<D, B, BK_MULTI, false>(a, tc, gi, G, sm, ring)) break;
             } else {
                 if (!team_sync(tc, a, &sm.flag) || !team_sync(tc, a, &sm.flag)) break;
             }
             if (!team_sync(tc, a, &sm.flag)) break;
             continue;
         }
+        constexpr bool CL = RUN == BK_CLUSTERS;
         if (G.mode != GM_BIDIR)
-            bk_group<D, B, BK_SINGLE>(a, tc, gi, G, sm, ring);
+            bk_group<D, B, BK_SINGLE, CL>(a, tc, gi, G, sm, ring);
         else if (a.searches[G.sbeg].pot)
-            bk_group<D, B, BK_BIDASTAR>(a, tc, gi, G, sm, ring);
+            bk_group<D, B, BK_BIDASTAR, CL>(a, tc, gi, G, sm, ring);
         else
-            bk_group<D, B, BK_BIDS>(a, tc, gi, G, sm, ring);
+            bk_group<D, B, BK_BIDS, CL>(a, tc, gi, G, sm, ring);
+        // the distances are clean, and the group's shared state read by all,
+        // before the next one starts
+        if (CL) cg::this_cluster().sync();
     }
 }
 
 // ---- host side ----
 constexpr size_t BK_SMEM_MAX = 227 * 1024;  // per CTA
 
-template <typename D, int B, bool TEAMS>
+template <typename D, int B, int RUN>
 static ppsp_status bucket_smem_attr() {
     static std::atomic<bool> done[SMEM_ATTR_DEVICES];
     int dev = 0;
     PPSP_CUDA_TRY(cudaGetDevice(&dev));
     if (dev >= 0 && dev < SMEM_ATTR_DEVICES && done[dev].load(std::memory_order_acquire)) return PPSP_OK;
-    PPSP_CUDA_TRY(cudaFuncSetAttribute(bucket_kernel<D, B, TEAMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PPSP_CUDA_TRY(cudaFuncSetAttribute(bucket_kernel<D, B, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)std::min<size_t>(bucket_smem_bytes<D>(RING_CAP_MAX), BK_SMEM_MAX)));
     if (dev >= 0 && dev < SMEM_ATTR_DEVICES) done[dev].store(true, std::memory_order_release);
     return PPSP_OK;
 }
 
-template <typename D, int B, bool TEAMS>
+// A launch of `grid` CTAs in clusters of `cluster`.
+struct BkClusterLaunch {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    BkClusterLaunch(u32 grid, u32 threads, size_t smem, u32 cluster, cudaStream_t stream) {
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cluster;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
+template <typename D, int B, int RUN>
 static ppsp_status bucket_launch_t(const EngineArgs& a, u32 grid, cudaStream_t stream) {
-    ppsp_status st = bucket_smem_attr<D, B, TEAMS>();
+    ppsp_status st = bucket_smem_attr<D, B, RUN>();
     if (st != PPSP_OK) return st;
     const size_t smem = bucket_smem_bytes<D>(a.ring_cap);
-    if (TEAMS) {
+    if (RUN == BK_TEAMS) {
         EngineArgs args = a;
         void* params[] = {&args};
-        PPSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bucket_kernel<D, B, TEAMS>, dim3(grid), dim3(B), params,
+        PPSP_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)bucket_kernel<D, B, RUN>, dim3(grid), dim3(B), params,
                                                   smem, stream));
+    } else if (RUN == BK_CLUSTERS) {
+        if (a.cluster < 1 || a.cluster > BK_CL_MAX || grid % a.cluster) return PPSP_ERR_INVALID_ARG;
+        BkClusterLaunch l(grid, B, smem, a.cluster, stream);
+        PPSP_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, bucket_kernel<D, B, RUN>, a));
     } else {
-        bucket_kernel<D, B, TEAMS><<<grid, B, smem, stream>>>(a);
+        bucket_kernel<D, B, RUN><<<grid, B, smem, stream>>>(a);
         PPSP_CUDA_TRY(cudaGetLastError());
     }
     return PPSP_OK;
 }
 
-template <typename D, bool TEAMS>
+template <typename D, int RUN>
 static ppsp_status bucket_launch(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream) {
     if (a.ring_cap < 1 || a.ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
-    if (block_threads == 256) return bucket_launch_t<D, 256, TEAMS>(a, grid, stream);
-    if (block_threads == 512) return bucket_launch_t<D, 512, TEAMS>(a, grid, stream);
-    if (block_threads == 1024) return bucket_launch_t<D, 1024, TEAMS>(a, grid, stream);
+    if (RUN != BK_CLUSTERS && block_threads == 256)
+        return bucket_launch_t<D, RUN == BK_CLUSTERS ? 512 : 256, RUN>(a, grid, stream);
+    if (block_threads == 512) return bucket_launch_t<D, 512, RUN>(a, grid, stream);
+    if (block_threads == 1024) return bucket_launch_t<D, 1024, RUN>(a, grid, stream);
     return PPSP_ERR_INVALID_ARG;
 }
 
-template <typename D, int B, bool TEAMS>
+// Resident CTAs per SM.
+template <typename D, int B, int RUN>
 static ppsp_status bucket_occ_t(int* bpsm, u32 ring_cap) {
-    ppsp_status st = bucket_smem_attr<D, B, TEAMS>();
+    ppsp_status st = bucket_smem_attr<D, B, RUN>();
     if (st != PPSP_OK) return st;
-    PPSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, bucket_kernel<D, B, TEAMS>, B,
+    PPSP_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(bpsm, bucket_kernel<D, B, RUN>, B,
                                                                 bucket_smem_bytes<D>(ring_cap)));
     return PPSP_OK;
 }
 
-template <typename D, bool TEAMS>
+template <typename D, int RUN>
 static ppsp_status bucket_occ(int block_threads, u32 ring_cap, int* bpsm) {
     if (ring_cap < 1 || ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
-    if (block_threads == 256) return bucket_occ_t<D, 256, TEAMS>(bpsm, ring_cap);
-    if (block_threads == 512) return bucket_occ_t<D, 512, TEAMS>(bpsm, ring_cap);
-    if (block_threads == 1024) return bucket_occ_t<D, 1024, TEAMS>(bpsm, ring_cap);
+    if (RUN != BK_CLUSTERS && block_threads == 256)
+        return bucket_occ_t<D, RUN == BK_CLUSTERS ? 512 : 256, RUN>(bpsm, ring_cap);
+    if (block_threads == 512) return bucket_occ_t<D, 512, RUN>(bpsm, ring_cap);
+    if (block_threads == 1024) return bucket_occ_t<D, 1024, RUN>(bpsm, ring_cap);
+    return PPSP_ERR_INVALID_ARG;
+}
+
+// Resident clusters of the whole device.
+template <typename D, int B>
+static ppsp_status bucket_clusters_t(u32 ring_cap, u32 cluster, int* clusters) {
+    ppsp_status st = bucket_smem_attr<D, B, BK_CLUSTERS>();
+    if (st != PPSP_OK) return st;
+    BkClusterLaunch l(cluster, B, bucket_smem_bytes<D>(ring_cap), cluster, 0);
+    PPSP_CUDA_TRY(cudaOccupancyMaxActiveClusters(clusters, bucket_kernel<D, B, BK_CLUSTERS>, &l.cfg));
+    return PPSP_OK;
+}
+
+template <typename D>
+static ppsp_status bucket_clusters(int block_threads, u32 ring_cap, u32 cluster, int* clusters) {
+    if (ring_cap < 1 || ring_cap > RING_CAP_MAX || cluster < 1 || cluster > BK_CL_MAX) return PPSP_ERR_INVALID_ARG;
+    if (block_threads == 512) return bucket_clusters_t<D, 512>(ring_cap, cluster, clusters);
+    if (block_threads == 1024) return bucket_clusters_t<D, 1024>(ring_cap, cluster, clusters);
     return PPSP_ERR_INVALID_ARG;
 }
 

@@ -1,5 +1,9 @@
 // Engine dispatch by distance width, and the small kernels of a plan run
 // (potential evaluation, result scatter).
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "engine_core.cuh"
 
 namespace ppsp {
@@ -13,11 +17,15 @@ ppsp_status engine_occupancy_u32(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u32_local(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status engine_occupancy_u64_local(int block_threads, u32 ring_cap, int* bpsm);
-// instantiated in bucket_{u32,u64}{,_teams}.cu
+// instantiated in bucket_{u32,u64}{,_teams,_clusters}.cu
 ppsp_status launch_bucket_u32(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
 ppsp_status launch_bucket_u64(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
 ppsp_status launch_bucket_u32_teams(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
 ppsp_status launch_bucket_u64_teams(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status launch_bucket_u32_clusters(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status launch_bucket_u64_clusters(const EngineArgs& a, int block_threads, u32 grid, cudaStream_t stream);
+ppsp_status resident_bucket_u32_clusters(int block_threads, u32 ring_cap, u32 cluster, int* clusters);
+ppsp_status resident_bucket_u64_clusters(int block_threads, u32 ring_cap, u32 cluster, int* clusters);
 ppsp_status occupancy_bucket_u32(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status occupancy_bucket_u64(int block_threads, u32 ring_cap, int* bpsm);
 ppsp_status occupancy_bucket_u32_teams(int block_threads, u32 ring_cap, int* bpsm);
@@ -28,6 +36,9 @@ ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads,
     const bool w32 = dist_bits == 32;
     if (kind == ENGINE_BUCKET)
         return w32 ? launch_bucket_u32(a, block_threads, grid, stream) : launch_bucket_u64(a, block_threads, grid, stream);
+    if (kind == ENGINE_BUCKET_CLUSTERS)
+        return w32 ? launch_bucket_u32_clusters(a, block_threads, grid, stream)
+                   : launch_bucket_u64_clusters(a, block_threads, grid, stream);
     if (kind == ENGINE_BUCKET_TEAMS)
         return w32 ? launch_bucket_u32_teams(a, block_threads, grid, stream)
                    : launch_bucket_u64_teams(a, block_threads, grid, stream);
@@ -37,23 +48,64 @@ ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads,
     return w32 ? launch_engine_u32(a, block_threads, grid, stream) : launch_engine_u64(a, block_threads, grid, stream);
 }
 
-ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms, EngineKind kind,
-                             u32 ring_cap) {
+// Occupancy answers, kept per device and configuration (a query to the driver
+// costs more than the rest of a small plan).
+namespace {
+struct OccCache {
+    std::mutex mu;
+    std::map<std::tuple<int, int, int, int, u32, u32>, int> got;
+} g_occ;
+
+template <typename F>
+ppsp_status occ_cached(int kind, int dist_bits, int block, u32 cap, u32 cluster, int* out, F ask) {
     int dev = 0;
     PPSP_CUDA_TRY(cudaGetDevice(&dev));
-    PPSP_CUDA_TRY(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+    const auto key = std::make_tuple(dev, kind, dist_bits, block, cap, cluster);
+    std::lock_guard<std::mutex> lk(g_occ.mu);
+    auto it = g_occ.got.find(key);
+    if (it == g_occ.got.end()) {
+        int v = 0;
+        const ppsp_status st = ask(dev, &v);
+        if (st != PPSP_OK) return st;
+        it = g_occ.got.emplace(key, v).first;
+    }
+    *out = it->second;
+    return PPSP_OK;
+}
+}  // namespace
+
+ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms, EngineKind kind,
+                             u32 ring_cap) {
+    ppsp_status st = occ_cached(-1, 0, 0, 0, 0, sms, [](int dev, int* v) {
+        PPSP_CUDA_TRY(cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev));
+        return PPSP_OK;
+    });
+    if (st != PPSP_OK) return st;
     const bool w32 = dist_bits == 32;
-    if (kind == ENGINE_BUCKET)
-        return w32 ? occupancy_bucket_u32(block_threads, ring_cap, blocks_per_sm)
-                   : occupancy_bucket_u64(block_threads, ring_cap, blocks_per_sm);
-    if (kind == ENGINE_BUCKET_TEAMS)
-        return w32 ? occupancy_bucket_u32_teams(block_threads, ring_cap, blocks_per_sm)
-                   : occupancy_bucket_u64_teams(block_threads, ring_cap, blocks_per_sm);
-    if (kind == ENGINE_LOCAL)
-        return w32 ? engine_occupancy_u32_local(block_threads, ring_cap, blocks_per_sm)
-                   : engine_occupancy_u64_local(block_threads, ring_cap, blocks_per_sm);
-    return w32 ? engine_occupancy_u32(block_threads, ring_cap, blocks_per_sm)
-               : engine_occupancy_u64(block_threads, ring_cap, blocks_per_sm);
+    return occ_cached(kind, dist_bits, block_threads, ring_cap, 0, blocks_per_sm, [=](int, int* v) {
+        switch (kind) {
+            case ENGINE_BUCKET:
+                return w32 ? occupancy_bucket_u32(block_threads, ring_cap, v)
+                           : occupancy_bucket_u64(block_threads, ring_cap, v);
+            case ENGINE_BUCKET_TEAMS:
+                return w32 ? occupancy_bucket_u32_teams(block_threads, ring_cap, v)
+                           : occupancy_bucket_u64_teams(block_threads, ring_cap, v);
+            case ENGINE_LOCAL:
+                return w32 ? engine_occupancy_u32_local(block_threads, ring_cap, v)
+                           : engine_occupancy_u64_local(block_threads, ring_cap, v);
+            default:
+                return w32 ? engine_occupancy_u32(block_threads, ring_cap, v)
+                           : engine_occupancy_u64(block_threads, ring_cap, v);
+        }
+    });
+}
+
+ppsp_status engine_clusters(int dist_bits, int block_threads, u32 ring_cap, u32 cluster, int* clusters) {
+    return occ_cached(ENGINE_BUCKET_CLUSTERS, dist_bits, block_threads, ring_cap, cluster, clusters,
+                      [=](int, int* v) {
+                          return dist_bits == 32 ? resident_bucket_u32_clusters(block_threads, ring_cap, cluster, v)
+                                                 : resident_bucket_u64_clusters(block_threads, ring_cap, cluster, v);
+                      });
 }
 
 // ---- adjacency blocks: one thread per record of a block; the thread of a

@@ -291,6 +291,31 @@ std::vector<SrcDir> sssp_sources(int strategy, bool directed, const std::vector<
 // 8- or 16-byte entries) takes 128 KB of an SM, whatever the CTAs' size.
 u32 bucket_cap(int block, int dist_bits) { return (u32)block / 4 / (dist_bits == 64 ? 2 : 1); }
 
+// Estimated device time (us) of a group of one or two searches on the bucketed
+// kernel with clusters of `cl` CTAs of 1,024 threads.  H: the queries' largest
+// heuristic distance in mean edge weights.  A step of e entries takes about
+// 2.2 + 0.0105 e us on one CTA, and a cluster splits the entries and pays 2 us
+// for its barrier and the others' states; a group takes about 1.2 H steps of c H entries (road-like
+// graphs of 512^2 to 4096^2, six random pairs or a 64-leaf star each: BiD-A*
+// c = 0.25 to 0.36, BiDS 1.05, ET and single-source 2.1 to 2.4).
+double bucket_group_us(u32 mode, bool pot, double H, double n, u32 cl) {
+    const double c = mode == GM_BIDIR ? (pot ? 0.3 : 1.05) : mode == GM_ASTAR ? 0.5 : 2.2;
+    const double steps = 1.2 * H + 20.0;
+    const double entries = std::min(c * H, 2.0 * n / steps);
+    return steps * (2.2 + (cl > 1 ? 2.0 : 0.0) + 0.0105 * entries / cl);
+}
+
+// Stepping increment of an A* group when no model is attached (mean edge
+// weight over this): along the shortest path the keys barely grow, so the
+// threshold runs ahead by one increment per hop, and a long path wants a small
+// one.  H: heuristic distance in mean edge weights.  One-directional A*, six
+// random pairs, w/4, w/8, w/16: 512^2 (H about 265) 12.2, 6.6, 11.3 ms; 1024^2
+// 57, 13.7, 16.1; 2048^2 1037, 224, 60.  BiD-A*, 1,000 pairs on 1024^2, w/4,
+// w/8, w/16, w/32: 139, 25.9, 16.2, 19.9 ms.
+double astar_divisor(bool bidir, double H) {
+    return bidir ? std::min(32.0, std::max(8.0, H / 32.0)) : std::min(32.0, std::max(6.0, H / 64.0));
+}
+
 // AUTO strategy: smallest number of targets that makes a source's queries
 // one multi-target search (ET / A* modes).
 constexpr u32 AUTO_MIN_TARGETS = 4;
@@ -567,7 +592,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     // ---- descriptors ----
     const u32 NG = (u32)gverts.size();
     std::vector<u32> uq_to_qe(U, NONE);
-    std::vector<double> gwork(NG, 1.0);
+    std::vector<double> gwork(NG, 1.0), gdist(NG, 0.0);  // estimated work; largest heuristic distance in mean weights
     for (u32 gi = 0; gi < NG; ++gi) {
         GroupDev G{};
         const auto& V = gverts[gi];
@@ -668,6 +693,10 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             work += (double)(hmax[i] + 1) * (double)(hmax[i] + 1) / (sssp ? 1.0 : 4.0);
         }
         gwork[gi] = work;
+        gdist[gi] = (double)*std::max_element(hmax.begin(), hmax.end()) / std::max(1e-9, g->info.w_mean);
+        if (o.delta == 0 && g->delta_model[o.mode] == nullptr &&
+            (G.mode == GM_ASTAR || (G.mode == GM_BIDIR && P->searches[G.sbeg].pot == 1)))
+            G.delta = std::max<u64>(1, (u64)std::llround((double)delta / astar_divisor(bidir, gdist[gi])));
         P->groups.push_back(G);
     }
     for (u64 q = 0; q < k; ++q)
@@ -823,7 +852,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     }
     if (tsize && (o.big_team_ctas || o.multi_potential || o.want_paths || strategy == PPSP_BATCH_PLAIN)) bucket = false;
     if (bucket) {
-        const EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
+        EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
         const u64 want = small.size() + (u64)tsize * big.size();  // CTAs that run everything at once
         int bb = o.block_threads;
         if (!bb) {
@@ -840,8 +869,40 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             bb = (want > 4 * (u64)sms && two <= g->device_mem / 4) ? 512 : 1024;
         }
         const u32 cap = o.ring_entries ? o.ring_entries : bucket_cap(bb, o.dist_bits);
+        // A cluster of CTAs per group where there are too few groups for the
+        // SMs and their steps are large, or the longest groups would outlast
+        // the rest: the smallest estimated time, by a tenth at least.
+        u32 cl = 1, ncl = 0;
+        if (!tsize && !o.want_paths && bb == 1024 && !small.empty()) {
+            double best = 0;
+            for (u32 k = 1; k <= 8; k *= 2) {
+                int nteams = sms;
+                if (k > 1) {
+                    st = engine_clusters(o.dist_bits, bb, cap, k, &nteams);
+                    if (st != PPSP_OK) return st;
+                }
+                if (o.max_ctas > 0) nteams = std::min<int>(nteams, o.max_ctas / (int)k);
+                if (strategy == PPSP_BATCH_PLAIN) nteams = std::min(nteams, 1);
+                if (nteams < 1) break;
+                double sum = 0, most = 0;
+                for (u32 gi : small) {
+                    const GroupDev& G = P->groups[gi];
+                    const double H = g->info.has_coords ? gdist[gi] : std::sqrt((double)n) / 2;
+                    const double us = bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k);
+                    sum += us;
+                    most = std::max(most, us);
+                }
+                const double us = std::max(sum / std::min<double>(nteams, (double)small.size()), most);
+                if (k == 1 || us < 0.9 * best) {
+                    best = us;
+                    cl = k;
+                    ncl = (u32)nteams;
+                }
+            }
+            if (cl > 1) kind = ENGINE_BUCKET_CLUSTERS;
+        }
         int bbpsm = 0, bsms = 0;
-        st = engine_occupancy(o.dist_bits, bb, &bbpsm, &bsms, kind, cap);
+        st = engine_occupancy(o.dist_bits, bb, &bbpsm, &bsms, cl > 1 ? ENGINE_BUCKET : kind, cap);
         if (st != PPSP_OK) return st;
         u32 res = (u32)(bbpsm * bsms);
         if (o.max_ctas > 0) res = std::min<u32>(res, (u32)o.max_ctas);
@@ -862,8 +923,11 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             const u32 ns = small.empty() ? (tsize ? 0u : 1u)
                                          : (strategy == PPSP_BATCH_PLAIN ? 1u : std::min<u32>(left, (u32)small.size()));
             teams.assign(nbt, {tsize, 0});
-            teams.insert(teams.end(), ns, {1, 1});
-            grid = nbt * tsize + ns;
+            teams.insert(teams.end(), cl > 1 ? std::min<u32>(ncl, (u32)small.size()) : ns, {cl, 1});
+            if (strategy == PPSP_BATCH_PLAIN && cl > 1) teams.resize(1);
+            grid = 0;
+            for (const TeamSpec& tm : teams) grid += tm.size;
+            P->args.cluster = cl;
             P->queue_items[0] = big;
             P->queue_items[1] = small;
             P->block = bb;

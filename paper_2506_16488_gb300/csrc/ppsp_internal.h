@@ -182,6 +182,7 @@ struct EngineArgs {
     u32 split;            // queue / bitmap path: rows longer than ROW_CHUNK are shared by the team
     u32 pull;             // queue / bitmap path: pull before push (App. B), undirected graphs
     u32 ring_cap;         // one-CTA path: shared-memory entries per bucket (1 .. 256)
+    u32 cluster;          // BUCKET_CLUSTERS: CTAs per group
     u32 debug;
     u64 spin_limit;
     u32* err;
@@ -214,8 +215,15 @@ void set_last_internal_error(const char* fmt, ...);
 // CTA per team with buckets in shared memory over the offsets (LOCAL), or the
 // same over the adjacency blocks of a graph of low degree: one CTA per group
 // of one or two searches (BUCKET), and one CTA per search of larger groups
-// (BUCKET_TEAMS).
-enum EngineKind { ENGINE_GENERAL = 0, ENGINE_LOCAL = 1, ENGINE_BUCKET = 2, ENGINE_BUCKET_TEAMS = 3 };
+// (BUCKET_TEAMS), or a cluster of CTAs per group of one or two searches
+// (BUCKET_CLUSTERS).
+enum EngineKind {
+    ENGINE_GENERAL = 0,
+    ENGINE_LOCAL = 1,
+    ENGINE_BUCKET = 2,
+    ENGINE_BUCKET_TEAMS = 3,
+    ENGINE_BUCKET_CLUSTERS = 4
+};
 
 // Launch a plan's kernel.  dist_bits selects the distance width.
 ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
@@ -226,6 +234,9 @@ ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads,
 constexpr u32 RING_CAP_DEFAULT = 64;
 ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms,
                              EngineKind kind = ENGINE_GENERAL, u32 ring_cap = RING_CAP_DEFAULT);
+
+// Resident clusters of the BUCKET_CLUSTERS kernel on the whole device.
+ppsp_status engine_clusters(int dist_bits, int block_threads, u32 ring_cap, u32 cluster, int* clusters);
 
 // Fill the adjacency blocks of one direction on the device (blk16 from
 // edges_pc, blk8 from edges; either may be null).  more[v]: record index of

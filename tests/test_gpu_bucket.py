@@ -136,3 +136,28 @@ def test_groups_of_several_searches(shape, bits):
                     for _ in range(2):  # the second batch finds the slots as the first left them
                         got = G.batch(p, mode=mode, strategy="multi", dist_bits=bits, **kw)
                         assert np.array_equal(got, want), (directed, mode, kw)
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("k", [1, 2, 5, 30])
+def test_clusters(k, bits):
+    """Few queries of large steps run on clusters of CTAs (2, 4 or 8 by the
+    number of queries): the same answers, hubs, overflow and far lists included."""
+    g, pairs = hub_graph(60000, DEGREES + (20000,), seed=38, extra=3)
+    pairs = np.r_[pairs[:k - 1], pairs[-1:]] if k > 1 else pairs[:1]
+    lost = np.array([[5, 60001]], dtype=np.uint32)
+    star = np.stack([np.full(12, pairs[0, 0]), np.arange(100, 112)], 1).astype(np.uint32)
+    d = one_way_graph(g, 0.2, seed=39)
+    for graph, directed in ((g, False), (d, True)):
+        want, far, st = (oracle.pairs(graph.offsets, graph.targets, graph.weights, p) for p in (pairs, lost, star))
+        for coords in (True, False):
+            with ppsp.Graph.from_csr(graph, undirected=not directed, with_coords=coords) as G:
+                for mode in MODES if coords else ("bids", "et"):
+                    for kw in ({}, {"delta": 1 << 40}, {"ring_entries": 1}, {"delta": 200, "ring_entries": 2},
+                               {"max_ctas": 3}):
+                        for _ in range(2):
+                            got = G.batch(pairs, mode=mode, strategy="plain_star", dist_bits=bits, **kw)
+                            assert np.array_equal(got, want), (directed, mode, kw)
+                    assert G.query(*pairs[0].tolist(), mode=mode, dist_bits=bits) == int(want[0])
+                    assert np.array_equal(G.batch(lost, mode=mode, strategy="plain_star", dist_bits=bits), far)
+                    assert np.array_equal(G.batch(star, mode=mode, strategy="vc", dist_bits=bits), st)
