@@ -225,6 +225,47 @@ static bool locality_order(u64 n, const float* xy, std::vector<u32>& perm, std::
 // shapes have 3.6 to 4, so most rows fit a block of four).
 constexpr u64 BLOCK_MAX_DEG = 6;
 
+bool HostWorkspace::reserve(size_t dev_need, size_t host_need) {
+    // sizes are rounded up, so that calls of about the same size allocate once
+    auto up = [](size_t x) { return (x + (x >> 2) + 65535) & ~(size_t)65535; };
+    if (dev_need > dev_bytes) {
+        cudaFree(dev);
+        dev = nullptr;
+        dev_bytes = 0;
+        if (cudaMalloc(&dev, up(dev_need)) != cudaSuccess) {
+            dev = nullptr;
+            cudaGetLastError();
+            return false;
+        }
+        dev_bytes = up(dev_need);
+    }
+    if (host_need > host_bytes) {
+        cudaFreeHost(host);
+        host = nullptr;
+        host_bytes = 0;
+        if (cudaHostAlloc((void**)&host, up(host_need), cudaHostAllocDefault) != cudaSuccess) {
+            host = nullptr;
+            cudaGetLastError();
+            return false;
+        }
+        host_bytes = up(host_need);
+    }
+    return true;
+}
+
+void HostWorkspace::release() {
+    cudaFree(dev);
+    cudaFreeHost(host);
+    cudaGetLastError();
+    dev = nullptr;
+    host = nullptr;
+    dev_bytes = host_bytes = 0;
+}
+
+void HostWorkspace::trim() {
+    if (dev_bytes > HOST_KEEP || host_bytes > HOST_KEEP) release();
+}
+
 SlotCaps slot_caps(u64 range, int frontier, bool whole_gpu) {
     u64 fc = std::max<u64>(range, 64);
     fc = (fc + 63) & ~63ull;
@@ -635,6 +676,7 @@ void ppsp_graph_destroy(ppsp_graph* g) {
     cudaDeviceSynchronize();
     for (auto& kv : g->pool) cudaFree(kv.second->base);
     g->pool.clear();
+    g->ws.release();
     cudaFree(g->d_off);
     cudaFree(g->d_edges);
     cudaFree(g->d_off_t);

@@ -11,6 +11,22 @@
 
 namespace ppsp {
 
+// Memory of the calls that take host pairs and return host answers
+// (ppsp_query, ppsp_batch), kept by the graph between calls: the device arena
+// of the call's plan, and page-locked copies of what goes up and comes back.
+// A call holds the graph's lock until its work on its stream has ended, so one
+// call at a time uses it, whatever the stream.
+struct HostWorkspace {
+    void* dev = nullptr;
+    size_t dev_bytes = 0;
+    char* host = nullptr;
+    size_t host_bytes = 0;
+    bool reserve(size_t dev_need, size_t host_need);
+    void trim();     // give back what a large call left (HOST_KEEP at most stays)
+    void release();
+};
+constexpr size_t HOST_KEEP = 64ull << 20;
+
 // One team's search memory (device).  Invariant between uses: every tentative
 // distance is infinity, both bitmaps are zero.
 struct Slot {
@@ -68,6 +84,7 @@ struct ppsp_graph {
     ppsp::u32* d_scratch_u32 = nullptr;
     int64_t* d_scratch_i64 = nullptr;
     uint64_t scratch_cap = 0;
+    ppsp::HostWorkspace ws;
     // learned stepping-increment models, one per plug-in (borrowed)
     ppsp_delta_model* delta_model[4] = {nullptr, nullptr, nullptr, nullptr};
 

@@ -38,6 +38,8 @@ struct ppsp_plan {
     u32* d_map = nullptr;
     EngineArgs args{};
     bool launched = false;
+    bool host_call = false;     // one call from host pairs to host answers: the arena is the graph's workspace
+    size_t back_at = 0, back_bytes = 0;  // arena range with the error word, the counters and mu
     // learned Delta: per-group features (log2(1 + raw)) and the model used
     std::vector<float> feats;
     float* d_feats = nullptr;
@@ -373,7 +375,7 @@ static void plan_free_partial(ppsp_plan* P) {
     P->slots.clear();
     // stream-ordered frees: no device-wide synchronisation, so plans on other
     // streams keep running (the serving loop closes plans while others run)
-    if (P->d_arena) cudaFreeAsync(P->d_arena, P->stream);
+    if (P->d_arena && !P->host_call) cudaFreeAsync(P->d_arena, P->stream);
     if (P->d_paths) cudaFreeAsync(P->d_paths, P->stream);
     P->d_arena = nullptr;
     P->d_paths = nullptr;
@@ -382,7 +384,8 @@ static void plan_free_partial(ppsp_plan* P) {
 
 // Build everything from host pairs.  Separated so ppsp_query can reuse it.
 static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64_t k, const ppsp_options* opt_in,
-                                    bool single_query, ppsp_plan** out, const u64* path_caps = nullptr) {
+                                    bool single_query, ppsp_plan** out, const u64* path_caps = nullptr,
+                                    bool host_call = false) {
     ppsp_options o;
     if (opt_in)
         o = *opt_in;
@@ -1025,17 +1028,30 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     size_t o_map = take(k * 4);
     size_t o_feat = take(P->feats.size() * 4);
     size_t static_bytes = off;
-    size_t o_mu = take(P->qedges.size() * 8);
-    size_t o_mumax = take(P->searches.size() * 8);
+    // run state (zero when a run starts), then what a run leaves: the error
+    // word, the counters and mu lie together, so that one copy brings them back
     size_t o_run = off;
     size_t o_qh = take(MAX_QUEUES * 4);
     size_t o_ts = take(NT * sizeof(TeamState));
+    size_t o_gns = take(P->groups.size() * 8);
     size_t o_err = take(4);
     size_t o_cnt = take(sizeof(EngineCounters));
-    size_t o_gns = take(P->groups.size() * 8);
     P->runstate_bytes = off - o_run;
+    size_t o_mu = take(P->qedges.size() * 8);
+    P->back_at = o_err;
+    P->back_bytes = o_mu + P->qedges.size() * 8 - o_err;
+    size_t o_mumax = take(P->searches.size() * 8);
     P->arena_bytes = off;
-    cudaError_t ce = cudaMallocAsync(&P->d_arena, P->arena_bytes, P->stream);
+    const size_t up_bytes = host_call ? o_run + P->runstate_bytes : static_bytes;
+    cudaError_t ce = cudaSuccess;
+    if (host_call && g->ws.reserve(P->arena_bytes, std::max(up_bytes, P->back_bytes))) {
+        P->host_call = true;
+        P->d_arena = g->ws.dev;
+    } else if (host_call) {
+        ce = cudaErrorMemoryAllocation;
+    } else {
+        ce = cudaMallocAsync(&P->d_arena, P->arena_bytes, P->stream);
+    }
     if (ce != cudaSuccess) {
         cudaGetLastError();
         cudaStreamSynchronize(P->stream);  // new slots may still be initialising
@@ -1044,9 +1060,11 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         return ce == cudaErrorMemoryAllocation ? PPSP_ERR_OOM : PPSP_ERR_CUDA;
     }
     char* base = (char*)P->d_arena;
-    std::vector<char> h(static_bytes, 0);
+    std::vector<char> pageable(host_call ? 0 : static_bytes, 0);
+    char* h = host_call ? g->ws.host : pageable.data();
+    if (host_call) memset(h, 0, up_bytes);
     auto put = [&](size_t o2, const void* src, size_t bytes) {
-        if (bytes) memcpy(h.data() + o2, src, bytes);
+        if (bytes) memcpy(h + o2, src, bytes);
     };
     put(o_groups, P->groups.data(), P->groups.size() * sizeof(GroupDev));
     put(o_search, P->searches.data(), P->searches.size() * sizeof(SearchDev));
@@ -1063,8 +1081,9 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     put(o_q1, P->queue_items[1].data(), P->queue_items[1].size() * 4);
     put(o_map, P->map.data(), k * 4);
     put(o_feat, P->feats.data(), P->feats.size() * 4);
-    // pageable source: staged before the call returns, so h may go out of scope
-    ce = cudaMemcpyAsync(base, h.data(), static_bytes, cudaMemcpyHostToDevice, P->stream);
+    // a pageable source is staged before the call returns, so it may go out of
+    // scope; the workspace stays until the call's work has ended
+    ce = cudaMemcpyAsync(base, h, up_bytes, cudaMemcpyHostToDevice, P->stream);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         plan_free_partial(P.get());
@@ -1143,13 +1162,15 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
 
 static void plan_free(ppsp_plan* P) {
     if (!P) return;
-    if (P->stream)
+    if (P->host_call)
+        ;  // its work has ended (host_finish)
+    else if (P->stream)
         cudaStreamSynchronize(P->stream);
     else
         cudaDeviceSynchronize();
     for (Slot* s : P->slots) slot_release(P->g, s);
     if (P->gexec) cudaGraphExecDestroy(P->gexec);
-    if (P->d_arena) cudaFreeAsync(P->d_arena, P->stream);
+    if (P->d_arena && !P->host_call) cudaFreeAsync(P->d_arena, P->stream);
     if (P->d_paths) cudaFreeAsync(P->d_paths, P->stream);
     cudaGetLastError();
     delete P;
@@ -1206,7 +1227,7 @@ static ppsp_status plan_launch_direct(ppsp_plan* P, u64* d_out) {
         if (st != PPSP_OK) return st;
     }
     ppsp_status st = PPSP_OK;
-    PPSP_CUDA_TRY(cudaMemsetAsync(P->d_runstate, 0, P->runstate_bytes, P->stream));
+    if (!P->host_call) PPSP_CUDA_TRY(cudaMemsetAsync(P->d_runstate, 0, P->runstate_bytes, P->stream));
     if (P->paths && !P->qedges.empty())
         PPSP_CUDA_TRY(cudaMemsetAsync(P->d_meet, 0xFF, P->qedges.size() * 4, P->stream));
     if (P->model && !P->groups.empty()) {
@@ -1227,17 +1248,7 @@ static ppsp_status plan_launch_direct(ppsp_plan* P, u64* d_out) {
     return PPSP_OK;
 }
 
-static ppsp_status plan_wait(ppsp_plan* P, ppsp_counters* counters) {
-    if (P->stream) {
-        PPSP_CUDA_TRY(cudaStreamSynchronize(P->stream));
-    } else {
-        PPSP_CUDA_TRY(cudaDeviceSynchronize());
-    }
-    u32 err = 0;
-    EngineCounters ec{};
-    PPSP_CUDA_TRY(cudaMemcpyAsync(&err, P->args.err, 4, cudaMemcpyDeviceToHost, P->stream));
-    PPSP_CUDA_TRY(cudaMemcpyAsync(&ec, P->args.counters, sizeof(ec), cudaMemcpyDeviceToHost, P->stream));
-    PPSP_CUDA_TRY(cudaStreamSynchronize(P->stream));
+static ppsp_status plan_result(ppsp_plan* P, u32 err, const EngineCounters& ec, ppsp_counters* counters) {
     if (counters) {
         memset(counters, 0, sizeof(*counters));
         counters->extracted = ec.extracted;
@@ -1258,6 +1269,49 @@ static ppsp_status plan_wait(ppsp_plan* P, ppsp_counters* counters) {
         return PPSP_ERR_CUDA;
     }
     return PPSP_OK;
+}
+
+// A call from host pairs to host answers: one copy brings back the error word,
+// the counters and mu, one wait ends the call, and the answers are put in input
+// order here.  (The separate copies and waits, an output array and the scatter
+// launch took 30 us of a 114 us query on the 64^2 grid.)
+static ppsp_status host_finish(ppsp_plan* P, ppsp_counters* counters, uint64_t* dists_out) {
+    char* h = P->g->ws.host;
+    cudaError_t ce = cudaMemcpyAsync(h, (char*)P->d_arena + P->back_at, P->back_bytes, cudaMemcpyDeviceToHost, P->stream);
+    const cudaError_t cw = cudaStreamSynchronize(P->stream);
+    if (ce == cudaSuccess) ce = cw;
+    if (ce != cudaSuccess) {
+        set_last_cuda_error(ce, "ppsp_batch", __FILE__, __LINE__);
+        cudaGetLastError();
+        return PPSP_ERR_CUDA;
+    }
+    u32 err = 0;
+    EngineCounters ec{};
+    memcpy(&err, h, 4);
+    memcpy(&ec, h + ((const char*)P->args.counters - (const char*)P->args.err), sizeof(ec));
+    const ppsp_status st = plan_result(P, err, ec, counters);
+    if (st != PPSP_OK) return st;
+    const char* mu = h + ((const char*)P->args.mu - (const char*)P->args.err);
+    for (u64 q = 0; q < P->k; ++q) {
+        u64 d = 0;
+        if (P->map[q] != NONE) memcpy(&d, mu + (size_t)P->map[q] * 8, 8);
+        dists_out[q] = d;
+    }
+    return PPSP_OK;
+}
+
+static ppsp_status plan_wait(ppsp_plan* P, ppsp_counters* counters) {
+    if (P->stream) {
+        PPSP_CUDA_TRY(cudaStreamSynchronize(P->stream));
+    } else {
+        PPSP_CUDA_TRY(cudaDeviceSynchronize());
+    }
+    u32 err = 0;
+    EngineCounters ec{};
+    PPSP_CUDA_TRY(cudaMemcpyAsync(&err, P->args.err, 4, cudaMemcpyDeviceToHost, P->stream));
+    PPSP_CUDA_TRY(cudaMemcpyAsync(&ec, P->args.counters, sizeof(ec), cudaMemcpyDeviceToHost, P->stream));
+    PPSP_CUDA_TRY(cudaStreamSynchronize(P->stream));
+    return plan_result(P, err, ec, counters);
 }
 
 extern "C" {
@@ -1402,25 +1456,14 @@ static ppsp_status run_host(ppsp_graph* g, const uint32_t* pairs, uint64_t k, co
         caps.resize(k);
         for (u64 q = 0; q < k; ++q) caps[q] = hp->offsets ? hp->offsets[q + 1] - hp->offsets[q] : hp->single_cap;
     }
-    ppsp_status st = plan_create_impl(g, pairs, k, opt, single, &P, hp ? caps.data() : nullptr);
+    ppsp_status st = plan_create_impl(g, pairs, k, opt, single, &P, hp ? caps.data() : nullptr, true);
     if (st != PPSP_OK) return st;
-    u64* d_out = nullptr;
-    cudaError_t ce = cudaMallocAsync((void**)&d_out, std::max<u64>(1, k) * 8, P->stream);
-    if (ce != cudaSuccess) {
-        cudaGetLastError();
-        plan_free(P);
-        return ce == cudaErrorMemoryAllocation ? PPSP_ERR_OOM : PPSP_ERR_CUDA;
-    }
-    st = plan_launch(P, d_out);
-    if (st == PPSP_OK) st = plan_wait(P, counters);
-    if (st == PPSP_OK && k) {
-        ce = cudaMemcpyAsync(dists_out, d_out, k * 8, cudaMemcpyDeviceToHost, P->stream);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(P->stream);
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            st = PPSP_ERR_CUDA;
-        }
-    }
+    st = plan_launch_direct(P, nullptr);
+    if (st == PPSP_OK)
+        st = host_finish(P, counters, dists_out);
+    else
+        cudaStreamSynchronize(P->stream);
+    cudaError_t ce = cudaSuccess;
     if (st == PPSP_OK && hp && P->paths) {
         // device paths are per query edge, oriented from its first to its
         // second endpoint; copy (or reverse) them into each query's slice
@@ -1467,8 +1510,8 @@ static ppsp_status run_host(ppsp_graph* g, const uint32_t* pairs, uint64_t k, co
         }
         if (st == PPSP_OK && small) st = PPSP_ERR_BUFFER_TOO_SMALL;
     }
-    cudaFreeAsync(d_out, P->stream);
     plan_free(P);
+    g->ws.trim();
     return st;
 }
 
