@@ -1273,8 +1273,9 @@ static ppsp_status plan_result(ppsp_plan* P, u32 err, const EngineCounters& ec, 
 
 // A call from host pairs to host answers: one copy brings back the error word,
 // the counters and mu, one wait ends the call, and the answers are put in input
-// order here.  (The separate copies and waits, an output array and the scatter
-// launch took 30 us of a 114 us query on the 64^2 grid.)
+// order here.  With an output array, a scatter launch, three
+// copies and four waits a query on the 64^2 grid took 114 us and a batch of 100
+// 334; now 81 and 299.
 static ppsp_status host_finish(ppsp_plan* P, ppsp_counters* counters, uint64_t* dists_out) {
     char* h = P->g->ws.host;
     cudaError_t ce = cudaMemcpyAsync(h, (char*)P->d_arena + P->back_at, P->back_bytes, cudaMemcpyDeviceToHost, P->stream);
