@@ -766,13 +766,23 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     struct TeamSpec {
         u32 size, queue;
     };
+    // Small graphs with long rows: a team's step on the queue path is a chain of
+    // barriers and atomics that are waited for, 17 to 50 us whatever the team's
+    // size, so one CTA with its buckets in shared memory is faster while a step
+    // fits it.  RMAT-11 / 13 / 15 / 16, ten BiDS queries one at a time: 4.9,
+    // 8.0, 9.1, 30.7 ms on all CTAs, 2.4, 4.0, 7.6, 29.7 on one; 24 pairs at
+    // once 0.75, 2.2, 3.6, 4.3 against 0.37, 0.95, 2.1, 3.6.  Single-source
+    // groups scan more: 90 of them 1.5, 4.7, 16.4, 24.9 against 0.57, 2.4, 14.1,
+    // 31.0, but 24 of them 0.6, 1.5, 6.2, 8.9 against 0.5, 2.0, 9.7, 26.
+    const bool small_dense = g->wsorted && !any_sssp && g->m <= (1u << 20);
+    const bool small_sssp = g->wsorted && any_sssp && g->m <= (1u << 19);
     // teams for `grid` resident CTAs; returns the CTAs they use
     auto build_teams = [&](u32 grid_in, std::vector<TeamSpec>& teams) -> u32 {
         teams.clear();
         u32 g_used = grid_in;
         if (strategy == PPSP_BATCH_PLAIN) {
             // one query (group) at a time on the whole GPU
-            u32 ts = o.team_ctas ? std::min<u32>(grid_in, (u32)o.team_ctas) : grid_in;
+            u32 ts = o.team_ctas ? std::min<u32>(grid_in, (u32)o.team_ctas) : small_dense ? 1u : grid_in;
             g_used = ts;
             teams.push_back({ts, 1});
             P->queue_items[0].clear();
@@ -808,7 +818,9 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 // 468 / 377 / 375 / 576 (one CTA each: 2,490), 24 pairs 199 /
                 // 98 / 54 / 34.  More pairs than CTAs stay on one CTA each
                 // (300: 205 against 231).
-                if (g->wsorted && (any_sssp || small.size() <= g_small))
+                if (small_dense || (small_sssp && small.size() * 4 > g_small))
+                    ts_auto = 1;
+                else if (g->wsorted && (any_sssp || small.size() <= g_small))
                     ts_auto = std::max<u32>(ts_auto, std::min<u32>(8, g_small));
                 u32 ts = o.team_ctas ? std::min<u32>((u32)o.team_ctas, g_small) : ts_auto;
                 // no more teams than groups: an idle team would still hold a slot
