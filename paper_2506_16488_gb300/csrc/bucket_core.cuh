@@ -165,7 +165,7 @@ __device__ __forceinline__ void bk_try_mu(const EngineArgs& a, const BkCtx<D>& c
 __device__ __forceinline__ float bk_h_est(int dx, int dy, float scale) {
     const float fx = (float)dx, fy = (float)dy;
     float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(fx * fx + fy * fy));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fx * fx + fy * fy));
     return y * scale;
 }
 static __device__ __noinline__ u64 bk_h_big(u64 d2, u32 shift) { return (u64)sqrt((double)d2) >> shift; }
@@ -276,14 +276,18 @@ __device__ __forceinline__ void bk_insert(BkCtx<D>& c, BkShared& sm, u32 f, u32 
     }
 }
 
-// Both searches' distances of v (pair), or the one search's.
+// The distance of <v, i> and, in a pair, the other search's (in the slot's
+// width: 64-bit copies of 32-bit distances cost registers and instructions).
 template <typename D, int KIND>
-__device__ __forceinline__ void bk_load(const BkCtx<D>& c, u32 v, u64& x0, u64& x1) {
+__device__ __forceinline__ void bk_load(const BkCtx<D>& c, u32 v, u32 i, D& own, D& oth) {
     if (!bk_one(KIND)) {
+        u64 x0, x1;
         ld_pair(c.dist, v, x0, x1);
+        own = (D)(i ? x1 : x0);
+        oth = (D)(i ? x0 : x1);
     } else {
-        x0 = ld_dist(c.dist + (KIND == BK_MULTI ? (((size_t)v << c.ks) | c.i0) : (size_t)v));
-        x1 = DT<D>::INF;
+        own = (D)ld_dist(c.dist + (KIND == BK_MULTI ? (((size_t)v << c.ks) | c.i0) : (size_t)v));
+        oth = (D)DT<D>::INF;
     }
 }
 
@@ -304,9 +308,10 @@ __device__ __forceinline__ D* bk_at(const BkCtx<D>& c, u32 f) {
 //
 // Measured (24-clique on the 1024^2 road graph, 11.8 M extractions): one team
 // of all CTAs on the queue / bitmap frontier, which inserts every waiting
-// entry again at every step, 244 ms; one CTA per search 41 ms (48 before the
-// row's loads were issued together; the fence is 8% of it), bound by the
-// latency of a step whose distances are a 128-byte row apart.
+// entry again at every step, 244 ms; one CTA per search 41 ms at the same
+// increment (48 before the row's loads were issued together; the fence is 8%
+// of it), 18.8 ms at the one the model now gives.  Bound by the latency of a
+// step whose distances are a 128-byte row apart.
 template <typename D>
 __device__ __forceinline__ void bk_update_one(const EngineArgs& a, BkShared& sm, u32 j, u64 o, u64 nd) {
     const u64 s = nd + o;
@@ -324,13 +329,16 @@ __device__ __forceinline__ void bk_update(const EngineArgs& a, const BkCtx<D>& c
         for (u32 p = 0; p < np; ++p) bk_update_one<D>(a, sm, sm.pj[p], ld_dist(row + sm.pj[p]), nd);
         return;
     }
-    // the whole row, 64 bytes in flight (a row has at least eight entries
-    // here); most of them are still infinite
-    constexpr u32 V = 16 / sizeof(D), CH = sizeof(D) == 4 ? 2 : 4;
+    // the whole row, 64 bytes in flight (32: 20.4 instead of 18.8 ms for the
+    // clique above); most entries are still infinite
+    constexpr u32 V = 16 / sizeof(D), CH = 4;
     for (u32 j0 = 0; j0 < (1u << c.ks); j0 += CH * V) {
         uint4 x[CH];
 #pragma unroll
-        for (u32 k = 0; k < CH; ++k) x[k] = __ldcg(reinterpret_cast<const uint4*>(row + j0 + k * V));
+        for (u32 k = 0; k < CH; ++k) {
+            x[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            if (j0 + k * V < (1u << c.ks)) x[k] = __ldcg(reinterpret_cast<const uint4*>(row + j0 + k * V));
+        }
 #pragma unroll
         for (u32 k = 0; k < CH; ++k) {
             const u32 j = j0 + k * V;
@@ -393,38 +401,37 @@ __device__ __forceinline__ BkRec bk_rec(const EngineArgs& a, bool pot, u32 dir, 
 // just read: they decide success (a concurrent smaller write only leaves a
 // stale entry behind, which extraction drops), so the write is not waited for.
 template <typename D, int KIND>
-__device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, u32 f, u64 d, const BkRec& r,
-                                         u64 x0, u64 x1) {
+__device__ __forceinline__ void bk_relax(const EngineArgs& a, BkCtx<D>& c, BkShared& sm, u32 f, D d, const BkRec& r,
+                                         D own, D oth) {
     constexpr u32 KS = bk_one(KIND) ? 0u : 1u;
     const u32 i = KS ? (f & 1u) : 0u;
-    const u64 nd = d + (u64)r.w;
+    const D nd = d + (D)r.w;
     ++c.c_e;
-    if (nd > DT<D>::MAXV) {
+    if (nd > (D)DT<D>::MAXV || nd < d) {
         // a distance that does not fit, unless the entry should have been
         // pruned (extraction does not test that)
         const int2 qv = a.g.pc ? __ldg(a.g.pc + (f >> KS)) : make_int2(0, 0);
         if (!pruned(bk_prune_value<D, KIND>(a, c, sm, i, qv, d), sm.bound)) atomicOr(a.err, ERRB_OVERFLOW);
         return;
     }
-    const u64 own = i ? x1 : x0, oth = i ? x0 : x1;
     if (nd >= own) return;
     const u32 v2 = r.v & ~BK_EXTRA, f2 = (v2 << KS) | i;
     if (KIND == BK_MULTI) {
-        if (amin_dist(bk_at<D, KIND>(c, f2), nd) <= nd) return;
+        if (amin_dist(bk_at<D, KIND>(c, f2), nd) <= (u64)nd) return;
         bk_update<D>(a, c, sm, v2, nd);
     } else {
         amin_dist(c.dist + f2, nd);
     }
     ++c.c_r;
     // the position in the touched list is asked for here and used at the end
-    const bool fresh = own == DT<D>::INF;
+    const bool fresh = own == (D)DT<D>::INF;
     u32 tpos = 0;
     if (fresh) {
         ++c.c_t;
         tpos = atomicAdd(&sm.tn, 1u);
     }
     if (!bk_one(KIND)) {
-        if (oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, nd + oth);
+        if (oth != (D)DT<D>::INF) bk_try_mu<D>(a, c, sm, (u64)nd + oth);
     } else if (KIND == BK_SINGLE && v2 == c.target) {
         bk_try_mu<D>(a, c, sm, nd);
     }
@@ -446,7 +453,7 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
     const u32 n = sm.n, s = sm.slot;
     for (u32 e1 = (CL ? sm.e0 : 0u) + (t >> 2); e1 < n; e1 += B / 4) {
         u32 f, e = e1;
-        u64 dins;
+        D dins;
         const typename BkEntry<D>::T* ring = c.ring;
         i64 ovf = (i64)((size_t)s * c.ob);
         if (CL) {
@@ -460,16 +467,16 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
         if (e < c.cap) {
             const typename BkEntry<D>::T x = ring[s * c.cap + e];
             f = (u32)x.x;
-            dins = x.y;
+            dins = (D)x.y;
         } else {
             f = __ldcg(sm.dev.of + ovf + (e - c.cap));
-            dins = ld_dist(reinterpret_cast<const D*>(sm.dev.od) + ovf + (e - c.cap));
+            dins = (D)ld_dist(reinterpret_cast<const D*>(sm.dev.od) + ovf + (e - c.cap));
         }
         const u32 extra = f & BK_EXTRA;
         f &= ~BK_EXTRA;
         const u32 v = f >> KS, i = KS ? (f & 1u) : 0u, dir = c.d0 | (i & c.dm);
-        u64 x0, x1;
-        bk_load<D, KIND>(c, v, x0, x1);
+        D d, oth;
+        bk_load<D, KIND>(c, v, i, d, oth);
         u32 rest = 0;   // continued edges after these four
         size_t at = (size_t)v * 4 + q4;
         if (extra) {
@@ -480,19 +487,18 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
             rest = rest > 4 ? rest - 4 : 0;
         }
         BkRec r = bk_rec<KIND>(a, pot, dir, at);
-        const u64 d = i ? x1 : x0;
         if (!bk_one(KIND) && q4 == 0 && !extra) {
             if (i) --c.dc1; else --c.dc0;  // the stored entry is consumed
         }
         if (d != dins) continue;  // stale: a smaller distance was inserted again
         if (q4 == 0 && !extra) {
             ++c.c_x;
-            const u64 oth = i ? x0 : x1;
-            if (!bk_one(KIND) && oth != DT<D>::INF) bk_try_mu<D>(a, c, sm, d + oth);
+            if (!bk_one(KIND) && oth != (D)DT<D>::INF) bk_try_mu<D>(a, c, sm, (u64)d + oth);
         }
         if (r.v < BLK_MORE) {
-            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
-            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+            D own;
+            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, i, own, oth);
+            bk_relax<D, KIND>(a, c, sm, f, d, r, own, oth);
         }
         if (rest) {
             bool mine = true;
@@ -510,8 +516,9 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
                         // no room: this lane scans them all
                         for (u32 j = 0; j < rest; ++j) {
                             r = bk_rec<KIND>(a, pot, dir, at + 4 + j);
-                            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
-                            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+                            D own;
+                            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, i, own, oth);
+                            bk_relax<D, KIND>(a, c, sm, f, d, r, own, oth);
                         }
                     }
                 }
@@ -520,8 +527,9 @@ __device__ __forceinline__ void bk_process(const EngineArgs& a, BkCtx<D>& c, BkS
             for (u32 j = q4; mine && j < rest; j += 4) {
                 at += 4;
                 r = bk_rec<KIND>(a, pot, dir, at);
-                bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
-                bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+                D own;
+                bk_load<D, KIND>(c, r.v & ~BK_EXTRA, i, own, oth);
+                bk_relax<D, KIND>(a, c, sm, f, d, r, own, oth);
             }
         }
     }
@@ -533,12 +541,12 @@ __device__ __forceinline__ void bk_deferred(const EngineArgs& a, BkCtx<D>& c, Bk
     const u32 nd = min(sm.ndef, BK_DEFER);
     for (u32 k = 0; k < nd; ++k) {
         const u32 f = sm.def_f[k], i = bk_one(KIND) ? 0u : (f & 1u);
-        const u64 d = sm.def_d[k];
+        const D d = (D)sm.def_d[k];
         for (u32 j = threadIdx.x; j < sm.def_cnt[k]; j += B) {
             const BkRec r = bk_rec<KIND>(a, pot, c.d0 | (i & c.dm), (size_t)sm.def_at[k] + j);
-            u64 x0, x1;
-            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, x0, x1);
-            bk_relax<D, KIND>(a, c, sm, f, d, r, x0, x1);
+            D own, oth;
+            bk_load<D, KIND>(c, r.v & ~BK_EXTRA, i, own, oth);
+            bk_relax<D, KIND>(a, c, sm, f, d, r, own, oth);
         }
     }
     __syncthreads();
