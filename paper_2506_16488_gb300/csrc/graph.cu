@@ -310,13 +310,11 @@ u64 slot_alloc_bytes(int dist_bits, u64 flat_cap, u32 qcap, u32 tcap, bool memo)
 ppsp_status slot_acquire(ppsp_graph* g, int dist_bits, u64 flat_cap, u32 qcap, u32 tcap, bool memo,
                          cudaStream_t stream, Slot** out) {
     SlotKey key{dist_bits, flat_cap, qcap, tcap, memo};
-    for (auto it = g->pool.lower_bound(key); it != g->pool.end(); ++it) {
-        Slot* s = it->second.get();
-        if (!s->busy && it->first.dist_bits == dist_bits && it->first.flat_cap >= flat_cap &&
-            it->first.qcap >= qcap && it->first.tcap >= tcap && it->first.flat_cap <= 2 * flat_cap + 4096 &&
-            (it->first.memo || !memo)) {
-            s->busy = true;
-            *out = s;
+    for (auto it = g->idle.lower_bound(key); it != g->idle.end(); ++it) {
+        if (it->first.dist_bits == dist_bits && it->first.flat_cap >= flat_cap && it->first.qcap >= qcap &&
+            it->first.tcap >= tcap && it->first.flat_cap <= 2 * flat_cap + 4096 && (it->first.memo || !memo)) {
+            *out = it->second;
+            g->idle.erase(it);
             return PPSP_OK;
         }
     }
@@ -368,15 +366,14 @@ ppsp_status slot_acquire(ppsp_graph* g, int dist_bits, u64 flat_cap, u32 qcap, u
     PPSP_CUDA_TRY(cudaMemsetAsync(s->dev.bm[0], 0, 2 * b_bm, stream));
     PPSP_CUDA_TRY(cudaMemsetAsync(s->dev.st, 0, b_st, stream));
     if (memo) PPSP_CUDA_TRY(cudaMemsetAsync(s->dev.memo, 0, L.b_memo, stream));  // 0 = no term memoized
-    s->busy = true;
+    s->key = key;
     *out = s.get();
-    g->pool.emplace(key, std::move(s));
+    g->pool.push_back(std::move(s));
     return PPSP_OK;
 }
 
 void slot_release(ppsp_graph* g, Slot* s) {
-    (void)g;
-    if (s) s->busy = false;
+    if (s) g->idle.emplace(s->key, s);
 }
 
 ppsp_status slot_scrub(Slot* s, cudaStream_t stream) {
@@ -674,7 +671,8 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
 void ppsp_graph_destroy(ppsp_graph* g) {
     if (!g) return;
     cudaDeviceSynchronize();
-    for (auto& kv : g->pool) cudaFree(kv.second->base);
+    for (auto& s : g->pool) cudaFree(s->base);
+    g->idle.clear();
     g->pool.clear();
     g->ws.release();
     cudaFree(g->d_off);

@@ -27,18 +27,6 @@ struct HostWorkspace {
 };
 constexpr size_t HOST_KEEP = 64ull << 20;
 
-// One team's search memory (device).  Invariant between uses: every tentative
-// distance is infinity, both bitmaps are zero.
-struct Slot {
-    void* base = nullptr;   // single allocation
-    size_t bytes = 0;
-    SlotDev dev{};
-    int dist_bits = 32;
-    u64 flat_cap = 0;
-    bool busy = false;
-    bool dirty = false;  // a failed run may have left it unclean: scrub before its next use
-};
-
 struct SlotKey {
     int dist_bits;
     u64 flat_cap;
@@ -49,6 +37,19 @@ struct SlotKey {
                std::tie(o.dist_bits, o.flat_cap, o.qcap, o.tcap, o.memo);
     }
 };
+
+// One team's search memory (device).  Invariant between uses: every tentative
+// distance is infinity, both bitmaps are zero.
+struct Slot {
+    void* base = nullptr;   // single allocation
+    size_t bytes = 0;
+    SlotDev dev{};
+    int dist_bits = 32;
+    u64 flat_cap = 0;
+    SlotKey key{};
+    bool dirty = false;  // a failed run may have left it unclean: scrub before its next use
+};
+
 
 }  // namespace ppsp
 
@@ -78,7 +79,8 @@ struct ppsp_graph {
     // caller id (both empty when the caller's order is kept)
     std::vector<ppsp::u32> perm, inv;
     // slot pool
-    std::multimap<ppsp::SlotKey, std::unique_ptr<ppsp::Slot>> pool;
+    std::vector<std::unique_ptr<ppsp::Slot>> pool;       // every slot of the graph
+    std::multimap<ppsp::SlotKey, ppsp::Slot*> idle;      // the ones no plan holds
     std::mutex mu;
     // scratch for small transfers (potential eval)
     ppsp::u32* d_scratch_u32 = nullptr;
