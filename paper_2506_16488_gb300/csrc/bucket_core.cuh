@@ -34,10 +34,12 @@
 // Measured against run_local (which took 17,000 cycles a step for one query
 // alone on the GPU: decision 3,400, extraction 4,100, relaxation 6,900, the
 // rest waiting; an L2 hit takes 290-360): one BiD-A* query on the 1024^2 road
-// graph 7.3 -> 2.4 ms (4.6 -> 1.1 ms over random pairs, where the start ran
-// the whole GPU), 1,000 queries on it 45.5 -> 16.4 ms, 2,048 on the 2048^2
+// graph 7.3 -> 2.4 ms (4.6 -> 1.1 ms over random pairs, where the queue path
+// took the whole GPU), 1,000 queries on it 45.5 -> 16.4 ms, 2,048 on the 2048^2
 // graph 228 -> 100 ms, 256 with 64-bit distances on the 4096^2 graph 255 ->
-// 136 ms.  DRAM traffic of the 2,048: 383 -> 213 GB.  What bounds it now: per
+// 136 ms.  With the longest pairs on more threads beside the rest (long_groups
+// in plan.cu) the 1,000 take 12.7 ms and the 256 82 to 93.  DRAM traffic of the
+// 2,048: 383 -> 213 GB.  What bounds it now: per
 // step and active warp about 500 instructions at 12.6 cycles each, of which a
 // third waits on global loads, a fifth on fixed-latency results and a seventh
 // on shared memory (one query alone); on a full GPU 0.46 of the issue slots
@@ -1040,7 +1042,7 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
     BkShared& sm = *reinterpret_cast<BkShared*>(smem_raw);
     unsigned char* ring = smem_raw + ((sizeof(BkShared) + 15) & ~(size_t)15);
     TeamCtx tc;
-    tc.team = RUN == BK_TEAMS ? a.cta_team[blockIdx.x] : RUN == BK_CLUSTERS ? blockIdx.x / a.cluster : blockIdx.x;
+    tc.team = RUN == BK_TEAMS ? a.cta_team[blockIdx.x] : RUN == BK_CLUSTERS ? blockIdx.x / a.cluster : a.team0 + blockIdx.x;
     tc.rank = RUN == BK_TEAMS ? blockIdx.x - a.team_first[tc.team] : RUN == BK_CLUSTERS ? blockIdx.x % a.cluster : 0u;
     tc.size = RUN == BK_TEAMS ? a.team_size[tc.team] : RUN == BK_CLUSTERS ? a.cluster : 1u;
     tc.ts = a.tstate + tc.team;
@@ -1048,6 +1050,7 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
     tc.expect = tc.size;
     tc.wait_shift = 4;
     const u32 qid = a.team_queue[tc.team];
+    if (RUN != BK_TEAMS && a.part == 1) cudaTriggerProgrammaticLaunchCompletion();
     if (threadIdx.x == 0) {
         SlotDev s = a.slots[tc.team];
         if (RUN != BK_CTAS && tc.size > 1) {
@@ -1114,6 +1117,8 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
         // before the next one starts
         if (CL) cg::this_cluster().sync();
     }
+    // what follows on the stream waits for the second launch only
+    if (RUN == BK_CTAS && a.part == 2) cudaGridDependencySynchronize();
 }
 
 // ---- host side ----
@@ -1162,6 +1167,19 @@ static ppsp_status bucket_launch_t(const EngineArgs& a, u32 grid, cudaStream_t s
         if (a.cluster < 1 || a.cluster > BK_CL_MAX || grid % a.cluster) return PPSP_ERR_INVALID_ARG;
         BkClusterLaunch l(grid, B, smem, a.cluster, stream);
         PPSP_CUDA_TRY(cudaLaunchKernelEx(&l.cfg, bucket_kernel<D, B, RUN>, a));
+    } else if (a.part == 2) {
+        // may start once every CTA of the first launch runs, on the SMs left
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(B);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        PPSP_CUDA_TRY(cudaLaunchKernelEx(&cfg, bucket_kernel<D, B, RUN>, a));
     } else {
         bucket_kernel<D, B, RUN><<<grid, B, smem, stream>>>(a);
         PPSP_CUDA_TRY(cudaGetLastError());

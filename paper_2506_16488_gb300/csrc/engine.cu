@@ -34,6 +34,21 @@ ppsp_status occupancy_bucket_u64_teams(int block_threads, u32 ring_cap, int* bps
 ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads, u32 grid,
                           cudaStream_t stream, EngineKind kind) {
     const bool w32 = dist_bits == 32;
+    if (kind == ENGINE_BUCKET && a.long_ctas && a.part == 0) {
+        // The longest groups on more threads each, the rest beside them.  Neither
+        // launch waits for the other's groups, so only the time depends on their
+        // running at once.
+        if (a.long_ctas >= grid || a.cluster < 1 || a.long_ctas % a.cluster) return PPSP_ERR_INVALID_ARG;
+        EngineArgs one = a, two = a;
+        one.part = 1;
+        one.ring_cap = a.long_cap;
+        two.part = 2;
+        two.team0 = a.long_ctas / a.cluster;
+        const ppsp_status st = launch_engine(one, dist_bits, 1024, a.long_ctas, stream,
+                                             a.cluster > 1 ? ENGINE_BUCKET_CLUSTERS : ENGINE_BUCKET);
+        return st == PPSP_OK ? launch_engine(two, dist_bits, block_threads, grid - a.long_ctas, stream, ENGINE_BUCKET)
+                             : st;
+    }
     if (kind == ENGINE_BUCKET)
         return w32 ? launch_bucket_u32(a, block_threads, grid, stream) : launch_bucket_u64(a, block_threads, grid, stream);
     if (kind == ENGINE_BUCKET_CLUSTERS)

@@ -297,14 +297,71 @@ u32 bucket_cap(int block, int dist_bits) { return (u32)block / 4 / (dist_bits ==
 // kernel with clusters of `cl` CTAs of 1,024 threads.  H: the queries' largest
 // heuristic distance in mean edge weights.  A step of e entries takes about
 // 2.2 + 0.0105 e us on one CTA, and a cluster splits the entries and pays 2 us
-// for its barrier and the others' states; a group takes about 1.2 H steps of c H entries (road-like
-// graphs of 512^2 to 4096^2, six random pairs or a 64-leaf star each: BiD-A*
-// c = 0.25 to 0.36, BiDS 1.05, ET and single-source 2.1 to 2.4).
-double bucket_group_us(u32 mode, bool pot, double H, double n, u32 cl) {
+// for its barrier and the others' states; a group takes about 1.2 H steps of
+// c H entries (road-like graphs of 512^2 to 4096^2, six random pairs or a
+// 64-leaf star each: BiD-A* c = 0.25 to 0.36, BiDS 1.05, ET and single-source
+// 2.1 to 2.4).  Searches with a potential take more steps per H the longer the
+// query (BiD-A*: 1.29 at a mean H of 483, 1.5 at 1974).
+// busy: what a cluster's entry costs more, over one CTA's.
+double bucket_group_us(u32 mode, bool pot, double H, double n, u32 cl, double busy = 0.0) {
     const double c = mode == GM_BIDIR ? (pot ? 0.3 : 1.05) : mode == GM_ASTAR ? 0.5 : 2.2;
-    const double steps = 1.2 * H + 20.0;
+    const double steps = 1.2 * H * (pot ? std::pow(std::max(H, 1.0) / 500.0, 0.15) : 1.0) + 20.0;
     const double entries = std::min(c * H, 2.0 * n / steps);
-    return steps * (2.2 + (cl > 1 ? 2.0 : 0.0) + 0.0105 * entries / cl);
+    return steps * (2.2 + (cl > 1 ? 2.0 : 0.0) + 0.0105 * entries * (1.0 / cl + (cl > 1 ? busy : 0.0)));
+}
+
+// Time of a group of 512 threads beside another one on the SM, over that of
+// 1,024 threads alone, for all groups and the longest: 1,000 BiD-A* queries on
+// the 1024^2 road graph 1.47, the 32 longest of them 1.59; one-directional A*
+// on 500^2 1.35 and 1.40.
+constexpr double GROUP_512 = 1.45, LONG_512 = 1.6;
+// What a cluster's entry costs more while the other SMs are busy, over one
+// CTA's entry: 256 BiD-A* queries on the 4096^2 graph, the longest on four CTAs
+// 83 ms where one takes 105.
+constexpr double CLUSTER_BUSY = 0.3;
+// A group takes up to this much longer than estimated.
+constexpr double LONG_SPREAD = 1.3;
+
+// Whether the longest BiD-A* pairs of a batch should start on more threads than
+// the rest, in a launch of their own, so that they do not outlast it.  Measured
+// in one launch / two: 1,000 queries on the 1024^2 road graph (two groups per
+// SM; the longest 15.6 ms, all together 11.8) 15.6 / 12.7 ms; 40, 150, 300, 700
+// on 2048^2 23.4, 32.3, 32.7, 60.4 / 16.7, 20.5, 24.1, 36.8; 256 with 64-bit
+// distances on 4096^2 105 / 82.  Not for other searches, whose estimates are
+// too rough and whose clusters slow one another more: 160 and 300 BiDS pairs
+// on 1024^2 10.2, 10.5 / 12.2, 12.9.
+// us: estimated times by CTAs per group (1, 2, 4, 8; 1,024 threads each),
+// longest first; per_sm: groups per SM of the rest; best: the estimate without.
+// Each count q of longest groups is tried with each size: the time is at least
+// that of its longest group, that of the rest's longest, and everything over
+// the SMs.
+struct LongGroups {
+    u32 groups = 0, cl = 1, teams = 0;
+};
+LongGroups long_groups(const std::vector<double> us[4], const u32 max_teams[4], u32 sms, u32 per_sm, double best) {
+    LongGroups r;
+    const double share = per_sm > 1 ? GROUP_512 : 1.0, tail = LONG_SPREAD * (per_sm > 1 ? LONG_512 : 1.0);
+    const u32 ng = (u32)us[0].size();
+    double all = 0;
+    for (double x : us[0]) all += x * share / per_sm;
+    best *= 0.95;
+    for (u32 c = per_sm > 1 ? 0 : 1; c < 4; ++c) {
+        if (us[c].empty()) continue;
+        double head = 0, longest = 0, rest = all;  // the longest groups' times, SM time of the rest
+        for (u32 q = 1; q < ng; ++q) {
+            head += us[c][q - 1];
+            longest = std::max(longest, us[c][q - 1]);
+            rest -= us[0][q - 1] * share / per_sm;
+            const u32 teams = std::min({q, max_teams[c], (3 * sms / 4) >> c});
+            if (teams == 0) break;
+            const double t = std::max({longest, head / teams, us[0][q] * tail, (head * (1u << c) + rest) / sms});
+            if (t < best) {
+                best = t;
+                r = {q, 1u << c, teams};
+            }
+        }
+    }
+    return r;
 }
 
 // Stepping increment of an A* group when no model is attached (mean edge
@@ -869,6 +926,8 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     if (bucket) {
         EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
         const u64 want = small.size() + (u64)tsize * big.size();  // CTAs that run everything at once
+        u64 small_range = 0;
+        for (u32 gi : small) small_range = std::max<u64>(small_range, n << P->groups[gi].kshift);
         int bb = o.block_threads;
         if (!bb) {
             // Two groups per SM (512 threads each) when there are enough of
@@ -877,17 +936,25 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             // finishes sooner.  Measured: 1,000 queries on the 1024^2 road
             // graph 16.4 against 17.6 ms, 2,048 on the 2048^2 one 100 against
             // 115 ms; 256 queries on the 4096^2 one 247 against 136 ms.
-            u64 range = 0;
-            for (u32 gi : small) range = std::max<u64>(range, n << P->groups[gi].kshift);
-            const SlotCaps sc = slot_caps(range, o.frontier, false);
+            const SlotCaps sc = slot_caps(small_range, o.frontier, false);
             const u64 two = 2ull * sms * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap);
             bb = (want > 4 * (u64)sms && two <= g->device_mem / 4) ? 512 : 1024;
         }
         const u32 cap = o.ring_entries ? o.ring_entries : bucket_cap(bb, o.dist_bits);
+        const u32 long_cap = o.ring_entries ? o.ring_entries : bucket_cap(1024, o.dist_bits);
         // A cluster of CTAs per group where there are too few groups for the
         // SMs and their steps are large, or the longest groups would outlast
         // the rest: the smallest estimated time, by a tenth at least.
+        auto group_us = [&](u32 gi, u32 k, double busy = 0.0) {
+            const GroupDev& G = P->groups[gi];
+            const double H = g->info.has_coords ? gdist[gi] : std::sqrt((double)n) / 2;
+            return bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k, busy);
+        };
         u32 cl = 1, ncl = 0;
+        double alone = 0;  // estimated time of the groups in one launch
+        bool all_pairs_pot = !tsize;  // BiD-A* pairs only
+        for (u32 gi : small)
+            all_pairs_pot = all_pairs_pot && P->groups[gi].mode == GM_BIDIR && P->searches[P->groups[gi].sbeg].pot;
         if (!tsize && !o.want_paths && bb == 1024 && !small.empty()) {
             double best = 0;
             for (u32 k = 1; k <= 8; k *= 2) {
@@ -901,9 +968,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 if (nteams < 1) break;
                 double sum = 0, most = 0;
                 for (u32 gi : small) {
-                    const GroupDev& G = P->groups[gi];
-                    const double H = g->info.has_coords ? gdist[gi] : std::sqrt((double)n) / 2;
-                    const double us = bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k);
+                    const double us = group_us(gi, k, all_pairs_pot && small.size() * k > (size_t)sms ? CLUSTER_BUSY : 0.0);
                     sum += us;
                     most = std::max(most, us);
                 }
@@ -915,6 +980,40 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 }
             }
             if (cl > 1) kind = ENGINE_BUCKET_CLUSTERS;
+            alone = best;
+        }
+        // The longest groups on more threads each, beside the rest.
+        LongGroups lg;
+        if (all_pairs_pot && (bb == 1024 || !o.block_threads) && !o.max_ctas &&
+            strategy != PPSP_BATCH_PLAIN && small.size() > 1) {
+            const u32 per_sm = bb == 512 ? 2 : 1;
+            std::vector<double> us[4];
+            u32 most[4] = {(u32)sms, 0, 0, 0};
+            for (u32 c = 0; c < (o.want_paths ? 1u : 4u); ++c) {
+                int nt = sms;
+                if (c) {
+                    st = engine_clusters(o.dist_bits, 1024, long_cap, 1u << c, &nt);
+                    if (st != PPSP_OK) return st;
+                }
+                most[c] = (u32)std::max(nt, 0);
+                for (u32 gi : small) us[c].push_back(group_us(gi, 1u << c, CLUSTER_BUSY));
+            }
+            if (bb == 512) {
+                double sum = 0, longest = 0;
+                for (double x : us[0]) {
+                    sum += x;
+                    longest = std::max(longest, x);
+                }
+                alone = std::max(LONG_512 * LONG_SPREAD * longest, GROUP_512 * sum / std::min<double>(2.0 * sms, (double)small.size()));
+            }
+            if (alone > 0) lg = long_groups(us, most, (u32)sms, per_sm, alone);
+            const SlotCaps sc = slot_caps(small_range, o.frontier, false);
+            const u64 slots = lg.teams + std::min<u64>(small.size() - lg.groups, (u64)per_sm * sms);
+            if (slots * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap) > g->device_mem / 2) lg = LongGroups();
+            if (lg.groups) {
+                kind = ENGINE_BUCKET;
+                cl = 1;
+            }
         }
         int bbpsm = 0, bsms = 0;
         st = engine_occupancy(o.dist_bits, bb, &bbpsm, &bsms, cl > 1 ? ENGINE_BUCKET : kind, cap);
@@ -940,11 +1039,21 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             teams.assign(nbt, {tsize, 0});
             teams.insert(teams.end(), cl > 1 ? std::min<u32>(ncl, (u32)small.size()) : ns, {cl, 1});
             if (strategy == PPSP_BATCH_PLAIN && cl > 1) teams.resize(1);
+            if (lg.groups) {
+                teams.assign(lg.teams, {lg.cl, 0});
+                teams.insert(teams.end(), std::min<u32>(res, (u32)small.size() - lg.groups), {1, 1});
+            }
             grid = 0;
             for (const TeamSpec& tm : teams) grid += tm.size;
-            P->args.cluster = cl;
+            P->args.cluster = lg.groups ? lg.cl : cl;
+            P->args.long_ctas = lg.teams * lg.cl;
+            P->args.long_cap = long_cap;
             P->queue_items[0] = big;
             P->queue_items[1] = small;
+            if (lg.groups) {  // no larger groups here
+                P->queue_items[0].assign(small.begin(), small.begin() + lg.groups);
+                P->queue_items[1].assign(small.begin() + lg.groups, small.end());
+            }
             P->block = bb;
             P->kind = kind;
             ring_cap = cap;
@@ -1011,6 +1120,17 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         const SlotCaps sc = slot_caps(range_q[teams[t].queue], o.frontier, teams[t].size == grid);
         Slot* s = nullptr;
         st = slot_acquire(g, o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap, P->memo, P->stream, &s);
+        if (st == PPSP_ERR_OOM && P->args.long_ctas && t > P->args.long_ctas / P->args.cluster) {
+            // two launches hold more slots than one would: run with fewer teams
+            grid -= (u32)teams.size() - t;
+            P->grid = grid;
+            P->cta_team.resize(grid);
+            P->team_first.resize(t);
+            P->team_size.resize(t);
+            P->team_queue.resize(t);
+            teams.resize(t);
+            break;
+        }
         if (st != PPSP_OK) {
             cudaStreamSynchronize(P->stream);  // new slots may still be initialising
             cudaGetLastError();

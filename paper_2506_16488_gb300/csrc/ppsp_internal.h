@@ -183,6 +183,11 @@ struct EngineArgs {
     u32 pull;             // queue / bitmap path: pull before push (App. B), undirected graphs
     u32 ring_cap;         // one-CTA path: shared-memory entries per bucket (1 .. 256)
     u32 cluster;          // BUCKET_CLUSTERS: CTAs per group
+    // BUCKET as two launches side by side (long_ctas > 0): first CTAs of 1,024
+    // threads, `cluster` of them per group, for the longest groups (queue 0)
+    u32 long_ctas, long_cap;  // its CTAs and ring_cap
+    u32 part;             // 1, 2: the first or second of the two launches, else 0
+    u32 team0;            // first team of the launch
     u32 debug;
     u64 spin_limit;
     u32* err;
