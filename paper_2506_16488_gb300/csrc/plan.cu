@@ -923,6 +923,18 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         bucket = bucket && P->groups[gi].layout == PPSP_LAYOUT_INTERLEAVED;
     }
     if (tsize && (o.big_team_ctas || o.multi_potential || o.want_paths || strategy == PPSP_BATCH_PLAIN)) bucket = false;
+    // An explicit increment far above the best one makes few steps of many
+    // thousand entries, which a large team shares better: few groups with one
+    // go to the queue path, as all did before.  One BiD-A* query at a time on
+    // the 2048^2 road graph with one mean weight: 1,950 ms on one CTA or a
+    // cluster, 44 to 66 on teams of 16, 12 to 16 on all CTAs.
+    if (bucket && o.delta && !o.team_ctas && (strategy == PPSP_BATCH_PLAIN || 2 * P->groups.size() <= grid_max)) {
+        double div = 0.5;
+        for (u32 gi : small)
+            if (P->searches[P->groups[gi].sbeg].pot)
+                div = std::max(div, astar_divisor(P->groups[gi].mode == GM_BIDIR, gdist[gi]) / 1.5);
+        if ((double)o.delta * div > g->info.w_mean) bucket = false;
+    }
     if (bucket) {
         EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
         const u64 want = small.size() + (u64)tsize * big.size();  // CTAs that run everything at once
