@@ -64,9 +64,10 @@ enum {
 enum { PPSP_UNDIRECTED = 1u, PPSP_KEEP_VERTEX_ORDER = 2u };
 
 /* Frontier representation policy (App. B "Sparse-Dense Optimization").
- * AUTO: a group run by one CTA keeps its frontier as Delta*-stepping buckets
- * in shared memory (overflow and far-ahead entries in the slot); a group run
- * by several CTAs uses a queue while the frontier is small and a bitmap once
+ * AUTO: a group run by one CTA or a cluster, and a Multi-BiDS group with one CTA
+ * per search, keeps its frontier as Delta*-stepping buckets in shared memory
+ * (overflow and far-ahead entries in the slot); a group run by a larger team
+ * (graphs with long rows, explicit team sizes) uses a queue while the frontier is small and a bitmap once
  * it exceeds (searches * n) / dense_den entries.  SPARSE / DENSE force the
  * queue / bitmap for every group. */
 enum { PPSP_FRONTIER_AUTO = 0, PPSP_FRONTIER_SPARSE = 1, PPSP_FRONTIER_DENSE = 2 };
@@ -145,8 +146,11 @@ typedef struct {
                                 path of undirected graphs: before an extracted vertex pushes,
                                 it pulls min over its neighbours x of d(x) + w(x, u); groups
                                 on one CTA and directed graphs ignore it.  Default 0         */
-    uint32_t ring_entries;   /* groups on one CTA: shared-memory entries per Delta-bucket of
-                                the frontier ring (32 buckets), 1..256; 0 = default (64).
+    uint32_t ring_entries;   /* groups with buckets in shared memory: entries per Delta-bucket
+                                of the frontier ring there, 1..256; 0 = default: 64 of 32
+                                buckets, or, on graphs of at most six adjacency entries per
+                                vertex, the CTA's threads / 4 (/ 8 with 64-bit distances) of
+                                64 buckets.
                                 Larger buckets stay out of the global overflow region; a
                                 smaller ring leaves more of the SM's L1 to the graph        */
     uint32_t multi_potential;/* BiD-A* Multi-BiDS groups: 1 = every shared search prunes with
@@ -215,6 +219,12 @@ const char* ppsp_last_error_detail(void);
  *            target: another 16m bytes, 32m for a directed graph), which the
  *            searches with a potential read instead of gathering the
  *            target's coordinates separately
+ *            A graph of at most six adjacency entries per vertex (and fewer
+ *            than 2^29 vertices) also gets one aligned block per vertex with its
+ *            first four edges, and the rest of longer rows: 36n bytes or more,
+ *            100n with coordinates, about twice that for a directed graph (none
+ *            where they would take more than an eighth of the free device
+ *            memory); device_bytes of ppsp_graph_info counts them
  *   flags    PPSP_UNDIRECTED: the CSR is symmetric with equal weights both ways
  *            (validated; the bidirectional modes search backwards on the same CSR).
  *            Without it the graph is directed: the library also keeps its
