@@ -656,8 +656,9 @@ __device__ __forceinline__ void flush_stage(GCtx<D>& c, Smem<B>& sm) {
 // End of the part of row [b0, b1) worth scanning from distance d: with rows
 // sorted by weight, the first edge whose candidate d + w is above the prune
 // bound (mu for searches joined by query edges, not mu / 2: a candidate of
-// that length can still be the middle edge of a path).  A longer candidate
-// can neither lower mu nor be inserted.  A row whose last candidate does not
+// that length can still be the middle edge of a path).  A longer candidate is
+// on no path shorter than the bound, whatever the potential (which prunes
+// entries, not distances), so it need not be written.  A row whose last candidate does not
 // fit the width keeps its full length, so that the overflow is reported.
 // On RMAT graphs most weights exceed what is left of the bound: RMAT-20, one
 // BiDS query 55.8 -> 10.2 M edges, the batch of 75 single-source groups 10.2 ->
@@ -754,6 +755,7 @@ template <typename D, int B>
 __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 cnt, bool sparse_src,
                               u32* bm_cur) {
     const u32 t = threadIdx.x;
+    const bool pull = a.pull && a.g.off == a.g.off_t;
     refresh_bounds<D, B>(a, c, sm);
     __syncthreads();
     u32 deg = 0;
@@ -802,7 +804,9 @@ __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 
                     update_bidir<D, B>(a, c, sm, v, i, d);
                 }
                 if (!pruned(pv, sm.bound[i])) {
-                    deg = cut_row<D, B>(a, sm, i, d, b0, b1) - b0;
+                    // the pull below may lower the distance, and edges too
+                    // long for this one reach then: whole rows with it
+                    deg = (pull ? b1 : cut_row<D, B>(a, sm, i, d, b0, b1)) - b0;
                     ++c.c_x;
                     if (a.split && c.slot.ocap && deg > ROW_CHUNK) {
                         // a long row: in pieces, for the whole team, after
@@ -837,7 +841,7 @@ __device__ void process_items(const EngineArgs& a, GCtx<D>& c, Smem<B>& sm, u32 
     sm.pre[t] = (t < cnt) ? excl : total;
     if (deg) write_owner<B>(sm, t, excl, deg);
     __syncthreads();
-    if (a.pull && a.g.off == a.g.off_t) {
+    if (pull) {
         // App. B, bidirectional relaxation: before pushing from u, pull
         // d(u) <- min(d(u), d(x) + w(x, u)) over its neighbours x (the same
         // adjacency on an undirected graph); every candidate is the length of
