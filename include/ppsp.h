@@ -352,6 +352,32 @@ ppsp_status ppsp_plan_features(const ppsp_plan* p, float* out, uint64_t cap, uin
 ppsp_status ppsp_plan_group_times(ppsp_plan* p, uint64_t* out_ns, uint64_t cap, uint64_t* ngroups);
 
 /*
+ * How a plan runs (host only; chosen when the plan is created).
+ *   kernel         PPSP_KERNEL_*
+ *   block_threads  threads per CTA (of the groups beside the longest ones)
+ *   ctas, teams    CTAs and teams of the plan
+ *   cluster        CTAs of a cluster (1: none); with long_groups, of the longest ones
+ *   long_groups    groups in a launch of their own beside the rest, 0: one launch
+ * Errors: INVALID_ARG.
+ */
+enum {
+    PPSP_KERNEL_GENERAL = 0,      /* teams of CTAs, queue / bitmap frontier               */
+    PPSP_KERNEL_LOCAL = 1,        /* one CTA per group, buckets, CSR rows                 */
+    PPSP_KERNEL_BUCKET = 2,       /* one CTA per group, buckets, adjacency blocks         */
+    PPSP_KERNEL_BUCKET_TEAMS = 3, /* the same, Multi-BiDS groups one CTA per search       */
+    PPSP_KERNEL_CLUSTERS = 4      /* adjacency blocks, a cluster of CTAs per group        */
+};
+typedef struct {
+    int32_t kernel;
+    int32_t block_threads;
+    uint32_t ctas, teams;
+    uint32_t cluster;
+    uint32_t long_groups;
+    uint32_t reserved[2];
+} ppsp_launch_shape;
+ppsp_status ppsp_plan_launch_shape(const ppsp_plan* p, ppsp_launch_shape* out);
+
+/*
  * Device memory of a plan (host outputs, each nullable):
  *   slot_bytes   search memory of its teams (one slot per team: distances,
  *                frontier bitmaps and queues, touched list, bucket overflow);

@@ -1542,6 +1542,18 @@ ppsp_status ppsp_batch_sources(const uint32_t* pairs, uint64_t k, int32_t strate
     return PPSP_OK;
 }
 
+ppsp_status ppsp_plan_launch_shape(const ppsp_plan* p, ppsp_launch_shape* out) {
+    if (!p || !out) return PPSP_ERR_INVALID_ARG;
+    *out = ppsp_launch_shape{};
+    out->kernel = (int32_t)p->kind;
+    out->block_threads = p->block;
+    out->ctas = p->grid;
+    out->teams = (u32)p->team_size.size();
+    out->cluster = std::max<u32>(1, p->args.cluster);
+    out->long_groups = p->args.long_ctas ? (u32)p->queue_items[0].size() : 0;
+    return PPSP_OK;
+}
+
 ppsp_status ppsp_plan_device_bytes(const ppsp_plan* p, uint64_t* slot_bytes, uint64_t* teams,
                                    uint64_t* other_bytes) {
     if (!p) return PPSP_ERR_INVALID_ARG;

@@ -223,11 +223,11 @@ void set_last_internal_error(const char* fmt, ...);
 // (BUCKET_TEAMS), or a cluster of CTAs per group of one or two searches
 // (BUCKET_CLUSTERS).
 enum EngineKind {
-    ENGINE_GENERAL = 0,
-    ENGINE_LOCAL = 1,
-    ENGINE_BUCKET = 2,
-    ENGINE_BUCKET_TEAMS = 3,
-    ENGINE_BUCKET_CLUSTERS = 4
+    ENGINE_GENERAL = PPSP_KERNEL_GENERAL,
+    ENGINE_LOCAL = PPSP_KERNEL_LOCAL,
+    ENGINE_BUCKET = PPSP_KERNEL_BUCKET,
+    ENGINE_BUCKET_TEAMS = PPSP_KERNEL_BUCKET_TEAMS,
+    ENGINE_BUCKET_CLUSTERS = PPSP_KERNEL_CLUSTERS
 };
 
 // Launch a plan's kernel.  dist_bits selects the distance width.

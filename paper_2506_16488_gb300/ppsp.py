@@ -98,6 +98,17 @@ class GraphInfo(ctypes.Structure):
         return {name: getattr(self, name) for name, _ in self._fields_}
 
 
+class LaunchShape(ctypes.Structure):
+    """ppsp_launch_shape: how a plan runs."""
+
+    _fields_ = [("kernel", ctypes.c_int32), ("block_threads", ctypes.c_int32), ("ctas", ctypes.c_uint32),
+                ("teams", ctypes.c_uint32), ("cluster", ctypes.c_uint32), ("long_groups", ctypes.c_uint32),
+                ("reserved", ctypes.c_uint32 * 2)]
+
+
+KERNELS = ("general", "local", "bucket", "bucket_teams", "clusters")
+
+
 class PPSPError(RuntimeError):
     """A non-OK ppsp_status; ``status`` holds the code."""
 
@@ -148,6 +159,7 @@ def load(build_if_missing: bool = False):
             "ppsp_plan_group_times": (S, [p, p, u64, p]),
             "ppsp_plan_uses_graph": (S, [p, p]),
             "ppsp_plan_device_bytes": (S, [p, p, p, p]),
+            "ppsp_plan_launch_shape": (S, [p, p]),
             "ppsp_slot_bytes": (S, [p, u32, i32, i32, p]),
             "ppsp_batch_sources": (S, [p, u64, i32, u32, p, p, p]),
             "ppsp_vertex_order": (S, [u64, p, p]),
@@ -459,6 +471,14 @@ class Plan:
         _check(load().ppsp_plan_device_bytes(self._handle(), ctypes.byref(sb), ctypes.byref(nt), ctypes.byref(ob)),
                "ppsp_plan_device_bytes")
         return {"slot_bytes": int(sb.value), "teams": int(nt.value), "other_bytes": int(ob.value)}
+
+    def launch_shape(self) -> dict:
+        """Kernel (KERNELS), threads, CTAs, teams, cluster size and groups in
+        a launch of their own (ppsp_plan_launch_shape)."""
+        ls = LaunchShape()
+        _check(load().ppsp_plan_launch_shape(self._handle(), ctypes.byref(ls)), "ppsp_plan_launch_shape")
+        d = {f: int(getattr(ls, f)) for f, _ in LaunchShape._fields_ if f != "reserved"}
+        return dict(d, kernel=KERNELS[d["kernel"]])
 
     def uses_graph(self) -> bool:
         """Whether the last run replayed a captured CUDA graph."""
