@@ -150,7 +150,8 @@ typedef struct {
                                 of the frontier ring there, 1..256; 0 = default: 64 of 32
                                 buckets, or, on graphs of at most six adjacency entries per
                                 vertex, the CTA's threads / 4 (/ 8 with 64-bit distances) of
-                                64 buckets.
+                                64 buckets (there at most 223 with 64-bit distances, what
+                                shared memory holds).
                                 Larger buckets stay out of the global overflow region; a
                                 smaller ring leaves more of the SM's L1 to the graph        */
     uint32_t multi_potential;/* BiD-A* Multi-BiDS groups: 1 = every shared search prunes with

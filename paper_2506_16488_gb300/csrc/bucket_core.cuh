@@ -1123,6 +1123,8 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
 
 // ---- host side ----
 constexpr size_t BK_SMEM_MAX = 227 * 1024;  // per CTA
+static_assert(bucket_smem_bytes<u32>(BK_RING_MAX_32) <= BK_SMEM_MAX && bucket_smem_bytes<u64>(BK_RING_MAX_64) <= BK_SMEM_MAX,
+              "the largest rings fit");
 
 template <typename D, int B, int RUN>
 static ppsp_status bucket_smem_attr() {

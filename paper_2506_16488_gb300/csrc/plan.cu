@@ -292,6 +292,11 @@ std::vector<SrcDir> sssp_sources(int strategy, bool directed, const std::vector<
 // Bucketed kernel: shared-memory entries per bucket.  The ring (64 buckets of
 // 8- or 16-byte entries) takes 128 KB of an SM, whatever the CTAs' size.
 u32 bucket_cap(int block, int dist_bits) { return (u32)block / 4 / (dist_bits == 64 ? 2 : 1); }
+// The same from the ring_entries option: at most what fits a CTA's shared memory.
+u32 bucket_cap(u32 ring_entries, int block, int dist_bits) {
+    if (!ring_entries) return bucket_cap(block, dist_bits);
+    return std::min(ring_entries, dist_bits == 64 ? BK_RING_MAX_64 : BK_RING_MAX_32);
+}
 
 // Estimated device time (us) of a group of one or two searches on the bucketed
 // kernel with clusters of `cl` CTAs of 1,024 threads.  H: the queries' largest
@@ -952,8 +957,8 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             const u64 two = 2ull * sms * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap);
             bb = (want > 4 * (u64)sms && two <= g->device_mem / 4) ? 512 : 1024;
         }
-        const u32 cap = o.ring_entries ? o.ring_entries : bucket_cap(bb, o.dist_bits);
-        const u32 long_cap = o.ring_entries ? o.ring_entries : bucket_cap(1024, o.dist_bits);
+        const u32 cap = bucket_cap(o.ring_entries, bb, o.dist_bits);
+        const u32 long_cap = bucket_cap(o.ring_entries, 1024, o.dist_bits);
         // A cluster of CTAs per group where there are too few groups for the
         // SMs and their steps are large, or the longest groups would outlast
         // the rest: the smallest estimated time, by a tenth at least.

@@ -237,6 +237,8 @@ ppsp_status launch_engine(const EngineArgs& a, int dist_bits, int block_threads,
 // Max resident CTAs of a kernel for a block size / distance width.
 // ring_cap: shared-memory entries per bucket of the one-CTA frontier.
 constexpr u32 RING_CAP_DEFAULT = 64;
+// Largest rings of the bucketed kernels (64 buckets; 64-bit entries take 16 bytes).
+constexpr u32 BK_RING_MAX_32 = 256, BK_RING_MAX_64 = 223;
 ppsp_status engine_occupancy(int dist_bits, int block_threads, int* blocks_per_sm, int* sms,
                              EngineKind kind = ENGINE_GENERAL, u32 ring_cap = RING_CAP_DEFAULT);
 
