@@ -2056,9 +2056,16 @@ __device__ __forceinline__ bool run_group(const EngineArgs& a, const TeamCtx& tc
 
         // entries of a tile: fewer than B while that leaves CTAs of the team
         // without one (a step of 8,000 entries on all 152 SMs is 16 tiles of
-        // 512), a warp's worth at least
+        // 512).  One tile a CTA, of 64 entries at least, since a second tile
+        // costs its barriers again: 24 BiDS pairs on a 700^2 road graph (300
+        // entries a step) on teams of four 11.5 ms with fixed tiles, 18.1 with
+        // two tiles a CTA of 32 at least, 11.8 with this; one query at a time on
+        // a nearest-neighbour graph (700 a step) on all CTAs 2.7, 1.4, 1.4 ms.
+        // Two tiles a CTA where rows are shared in pieces (RMAT-18: 31.6 ms
+        // against 32.7).
         if (!dense_cur) {
-            const u32 ts = tc.size == 1 ? (u32)B : min((u32)B, max(32u, count / (2 * tc.size)));
+            u32 ts = B;
+            if (tc.size > 1) ts = min(ts, a.split ? max(32u, count / (2 * tc.size)) : max(64u, count / tc.size));
             const u32 nt = (count + ts - 1) / ts;
             u32 local = tc.rank;
             for (;;) {
