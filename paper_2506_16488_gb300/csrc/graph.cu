@@ -225,6 +225,58 @@ static bool locality_order(u64 n, const float* xy, std::vector<u32>& perm, std::
 // shapes have 3.6 to 4, so most rows fit a block of four).
 constexpr u64 BLOCK_MAX_DEG = 6;
 
+// How fast the graph's neighbourhoods grow: breadth-first balls of up to
+// GROWTH_BALL vertices around GROWTH_STARTS vertices of at least average degree
+// spread over the ids (balls of a small component left out), by majority.  A
+// ball of L levels has at most 14 L^2 vertices on the shapes whose searches have
+// many short steps: 2 L^2 on a grid, 8 L^2 on road-like grids with shortcuts (33
+// to 60 levels for 8,192 vertices), 4 L on a chain.  On a power-law graph (2 to 6
+// levels) or a grid of three dimensions (18) a search has few steps of very many
+// entries, the opposite of what the kernels over adjacency blocks are made for.  From a sixteenth to a half of a ball the
+// levels double in three dimensions and grow by a third to a half where growth is
+// exponential.  Takes 0.2 to 3 ms.
+constexpr u64 GROWTH_BALL = 8192;
+constexpr u32 GROWTH_STARTS = 3;
+static Growth graph_growth(u64 n, const u64* off, const u32* tgt) {
+    struct Ball {
+        u64 size, levels;
+        bool exponential;
+    } got[GROWTH_STARTS];
+    std::vector<u32> seen(n, 0), ball;
+    std::vector<u64> upto;  // vertices of the ball's first levels
+    u64 largest = 0;
+    for (u32 k = 0; k < GROWTH_STARTS; ++k) {
+        u64 start = n * (2 * k + 1) / (2 * GROWTH_STARTS);
+        while ((off[start + 1] - off[start]) * n < off[n]) start = start + 1 < n ? start + 1 : 0;
+        ball.assign(1, (u32)start);
+        seen[ball[0]] = k + 1;
+        upto.assign(1, 1);
+        u64 head = 0;
+        while (head < ball.size() && ball.size() < GROWTH_BALL) {
+            const u64 end = ball.size();
+            for (; head < end && ball.size() < GROWTH_BALL; ++head)
+                for (u64 e = off[ball[head]]; e < off[ball[head] + 1] && ball.size() < GROWTH_BALL; ++e)
+                    if (seen[tgt[e]] != k + 1) {
+                        seen[tgt[e]] = k + 1;
+                        ball.push_back(tgt[e]);
+                    }
+            upto.push_back(ball.size());
+        }
+        auto levels_to = [&](u64 size) {
+            return (u64)(std::lower_bound(upto.begin(), upto.end(), size) - upto.begin());
+        };
+        got[k] = {ball.size(), upto.size() - 1,
+                  4 * levels_to(ball.size() / 2) < 7 * levels_to(ball.size() / 16)};
+        largest = std::max<u64>(largest, ball.size());
+    }
+    u32 count[3] = {0, 0, 0};
+    for (const Ball& b : got)
+        if (2 * b.size >= largest)
+            ++count[14 * b.levels * b.levels >= b.size ? GROWTH_PLANE : b.exponential ? GROWTH_RANDOM : GROWTH_WIDE];
+    if (count[GROWTH_PLANE] >= count[GROWTH_WIDE] + count[GROWTH_RANDOM]) return GROWTH_PLANE;
+    return count[GROWTH_RANDOM] > count[GROWTH_WIDE] ? GROWTH_RANDOM : GROWTH_WIDE;
+}
+
 bool HostWorkspace::reserve(size_t dev_need, size_t host_need) {
     // sizes are rounded up, so that calls of about the same size allocate once
     auto up = [](size_t x) { return (x + (x >> 2) + 65535) & ~(size_t)65535; };
@@ -472,6 +524,7 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
     // the first edge that reaches it (cut_row in engine_core.cuh).  Nothing else
     // depends on the order within a row.
     g->wsorted = m > BLOCK_MAX_DEG * n;
+    g->growth = graph_growth(n, offsets, targets);
     auto sort_rows = [](u64 rows, const auto* off, uint2* ed) {
         parallel_for(rows, [&](u64 lo, u64 hi, unsigned) {
             for (u64 v = lo; v < hi; ++v)
@@ -615,9 +668,12 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
         }
     }
     // Adjacency blocks for the bucketed kernel: graphs of average degree at
-    // most BLOCK_MAX_DEG.  They are left out, and plans run over the offsets, when they would take more than an
-    // eighth of the free device memory or a record index 32 bits.
-    if (m <= BLOCK_MAX_DEG * n && n < (1ull << 29)) {
+    // most BLOCK_MAX_DEG.  They are left out, and plans run over the offsets, on
+    // graphs whose plans never take that kernel (blocks_pay in plan.cu), and when
+    // they would take more than an eighth of the free device memory or a record
+    // index 32 bits.
+    if (m <= BLOCK_MAX_DEG * n && n < (1ull << 29) &&
+        (g->growth == GROWTH_PLANE || n <= BLOCK_SMALL_N || dmax <= BLOCK_MAX_ROW)) {
         const u32 dirs = info.undirected ? 1 : 2;
         std::vector<u32> more[2];  // record index of the continued edges, per direction
         u64 recs[2] = {0, 0};

@@ -27,6 +27,13 @@ struct HostWorkspace {
 };
 constexpr size_t HOST_KEEP = 64ull << 20;
 
+// How fast a graph's neighbourhoods grow (graph_growth).
+enum Growth {
+    GROWTH_PLANE = 0,  // as in the plane or slower
+    GROWTH_WIDE = 1,   // faster
+    GROWTH_RANDOM = 2  // exponentially, as in a random graph
+};
+
 struct SlotKey {
     int dist_bits;
     u64 flat_cap;
@@ -64,6 +71,7 @@ struct ppsp_graph {
     uint2* d_edges_t = nullptr;
     int2* d_pc = nullptr;
     bool wsorted = false;          // rows sorted by weight on the device
+    ppsp::Growth growth = ppsp::GROWTH_PLANE;  // of its neighbourhoods
     uint64_t device_mem = 0;       // total memory of the device
     void* d_blocks = nullptr;      // adjacency blocks (GraphDev::blk8 ...), one allocation, or null
     uint2* d_blk8 = nullptr;

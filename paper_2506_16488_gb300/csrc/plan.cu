@@ -380,6 +380,26 @@ double astar_divisor(bool bidir, double H) {
     return bidir ? std::min(32.0, std::max(8.0, H / 32.0)) : std::min(32.0, std::max(6.0, H / 64.0));
 }
 
+// Whether a plan takes the kernels over adjacency blocks (on a graph that has
+// them).  Where neighbourhoods grow as in the plane, always.  Elsewhere the steps
+// of a search have very many entries, which outgrow a CTA's buckets and their
+// overflow regions, so large graphs, graphs with long rows and few groups, which
+// have many CTAs each on the queue path, keep the other kernels.  Measured, queue
+// path or run_local / this kernel: one query at a time, ET on a random graph of
+// 2^20 vertices (average degree 5.5) 1.3 / 132 ms, BiDS on RMAT-20 with edge
+// factor 3 6.2 / 165, BiDS on a 100^3 grid 1.4 / 61; 200 at once: ET on random
+// graphs of 2^15, 2^16, 2^17, 2^20 vertices 21, 68, 101, 1,490 / 2.5, 15, 37,
+// 3,860 ms, BiDS on RMAT-13 and -15 with edge factor 3 1.4, 5.8 / 1.9, 10.2.
+// Bidirectional searches of a random graph settle about sqrt(n) vertices and
+// are short whatever its size: 24 BiDS pairs on 2^15, 2^18, 2^20 vertices 0.22,
+// 0.32, 0.49 / 0.09, 0.17, 0.32; 1,000 pairs on 2^17 vertices 1.1 / 2.7.
+// ctas: CTAs that run everything at once; one: one CTA per group.
+bool blocks_pay(const ppsp_graph* g, bool all_bidir, bool one, bool pairs_only, u64 ctas, u32 sms) {
+    if (g->growth == GROWTH_PLANE || g->n <= BLOCK_SMALL_N) return true;
+    if (g->info.deg_max > BLOCK_MAX_ROW) return false;
+    return (g->growth == GROWTH_RANDOM && all_bidir && ctas <= sms) || (one && pairs_only && g->n <= (1u << 16));
+}
+
 // AUTO strategy: smallest number of targets that makes a source's queries
 // one multi-target search (ET / A* modes).
 constexpr u32 AUTO_MIN_TARGETS = 4;
@@ -804,8 +824,13 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     // ---- launch shape ----
     // teams of several CTAs: 512 threads (128 registers), or 1,024 (64) where
     // rows are long and the edge loop, which needs few registers, dominates
-    // (RMAT-20: 75 groups 174 against 130 ms on teams of eight)
-    int block = o.block_threads ? o.block_threads : (g->wsorted ? 1024 : 512);
+    // (RMAT-20: 75 groups 174 against 130 ms on teams of eight).  Not on
+    // graphs with long rows that grow as in the plane (nearest-neighbour
+    // graphs), whose steps are short (2^18 vertices, eight neighbours each: 8
+    // BiDS queries one at a time 13.8 against 11.1 ms, 24 pairs 4.8 on 1,024
+    // threads and teams of eight against 4.0)
+    const bool hubs = g->wsorted && g->growth != GROWTH_PLANE;
+    int block = o.block_threads ? o.block_threads : (hubs ? 1024 : 512);
     int bpsm = 0, sms = 0;
     u32 ring_cap = o.ring_entries ? o.ring_entries : RING_CAP_DEFAULT;
     st = engine_occupancy(o.dist_bits, block, &bpsm, &sms, ENGINE_GENERAL, ring_cap);
@@ -871,7 +896,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 // fewer groups than CTAs: give each group a team of several CTAs
                 u32 ts_auto = 1;
                 while (ts_auto * 2 <= 32 && (u64)ts_auto * 2 * small.size() <= g_small) ts_auto *= 2;
-                // Graphs with long rows (RMAT shapes): eight CTAs at least,
+                // Graphs with long rows and hubs (RMAT shapes): eight CTAs at least,
                 // which take the groups in turn, longest first: a group's
                 // steps are large enough to share, and the longest one (a
                 // search with many targets) no longer outlasts the rest.
@@ -882,7 +907,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 // (300: 205 against 231).
                 if (small_dense || (small_sssp && small.size() * 4 > g_small))
                     ts_auto = 1;
-                else if (g->wsorted && (any_sssp || small.size() <= g_small))
+                else if (hubs && (any_sssp || small.size() <= g_small))
                     ts_auto = std::max<u32>(ts_auto, std::min<u32>(8, g_small));
                 u32 ts = o.team_ctas ? std::min<u32>((u32)o.team_ctas, g_small) : ts_auto;
                 // no more teams than groups: an idle team would still hold a slot
@@ -928,6 +953,14 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         bucket = bucket && P->groups[gi].layout == PPSP_LAYOUT_INTERLEAVED;
     }
     if (tsize && (o.big_team_ctas || o.multi_potential || o.want_paths || strategy == PPSP_BATCH_PLAIN)) bucket = false;
+    if (bucket) {
+        bool all_bidir = true;
+        for (const GroupDev& G : P->groups) all_bidir = all_bidir && G.mode == GM_BIDIR;
+        const bool plain = strategy == PPSP_BATCH_PLAIN;
+        const u64 ctas = plain ? std::max<u32>(1, tsize) : small.size() + (u64)tsize * big.size();
+        const bool one = !plain && (o.team_ctas == 1 || 2 * P->groups.size() > grid_max);
+        bucket = blocks_pay(g, all_bidir, one, tsize == 0, ctas, (u32)sms);
+    }
     // An explicit increment far above the best one makes few steps of many
     // thousand entries, which a large team shares better: few groups with one
     // go to the queue path, as all did before.  One BiD-A* query at a time on

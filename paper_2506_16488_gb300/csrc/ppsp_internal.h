@@ -33,6 +33,11 @@ constexpr u32 ROW_CHUNK = 2048;
 constexpr int KMAX = 64;          // searches per group (query-graph vertices)
 constexpr int MAX_QUEUES = 2;     // group queues: 0 = multi-search groups, 1 = pairs/singles
 
+// Graphs that do not grow as in the plane take the kernels over adjacency
+// blocks up to BLOCK_SMALL_N vertices, or with no row longer than BLOCK_MAX_ROW
+// (blocks_pay in plan.cu).
+constexpr u64 BLOCK_SMALL_N = 4096, BLOCK_MAX_ROW = 64;
+
 // Targets that are no vertex (with blocks, ids are below 2^30), see
 // GraphDev::blk8.
 constexpr u32 BLK_NONE = ~0u;
