@@ -980,15 +980,18 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         for (u32 gi : small) small_range = std::max<u64>(small_range, n << P->groups[gi].kshift);
         int bb = o.block_threads;
         if (!bb) {
-            // Two groups per SM (512 threads each) when there are enough of
-            // them to fill both and the slots of twice the teams leave most of
+            // Two groups per SM (512 threads each) when enough of them run at
+            // once to fill both (not one at a time, nor on max_ctas CTAs that
+            // fit the SMs) and the slots of twice the teams leave most of
             // the memory free; otherwise one group of 1,024 threads, which
             // finishes sooner.  Measured: 1,000 queries on the 1024^2 road
             // graph 16.4 against 17.6 ms, 2,048 on the 2048^2 one 100 against
             // 115 ms; 256 queries on the 4096^2 one 247 against 136 ms.
             const SlotCaps sc = slot_caps(small_range, o.frontier, false);
             const u64 two = 2ull * sms * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap);
-            bb = (want > 4 * (u64)sms && two <= g->device_mem / 4) ? 512 : 1024;
+            const bool both = strategy != PPSP_BATCH_PLAIN && want > 4 * (u64)sms &&
+                              (!o.max_ctas || 2 * (u64)o.max_ctas > 3 * (u64)sms);
+            bb = (both && two <= g->device_mem / 4) ? 512 : 1024;
         }
         const u32 cap = bucket_cap(o.ring_entries, bb, o.dist_bits);
         const u32 long_cap = bucket_cap(o.ring_entries, 1024, o.dist_bits);

@@ -1,0 +1,38 @@
+"""Rules of a plan's launch: CTA size and clusters where groups run one at a
+time, on few CTAs or on explicit sizes, team_ctas = 1, little device memory,
+and increments and estimates without a usable potential."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2506_16488_gb300 import ppsp
+from workloads import CSRGraph, clique_pairs, csr_from_undirected, grid_graph, random_pairs, road_like_graph
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def road():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    g = road_like_graph(700, seed=61)
+    with ppsp.Graph.from_csr(g) as G:
+        yield g, G
+
+
+def shape_of(G, pairs, **kw):
+    with G.plan(pairs, **kw) as p:
+        return p.launch_shape()
+
+
+@pytest.mark.parametrize("mode", ["et", "bids", "bidastar"])
+def test_one_group_at_a_time_gets_whole_ctas(road, mode):
+    g, G = road
+    pairs = random_pairs(g, 700, 62)
+    few, many = (shape_of(G, pairs[:k], mode=mode, strategy="plain") for k in (10, 700))
+    assert many["block_threads"] == 1024 and many["cluster"] == few["cluster"], (few, many)
+    lane = shape_of(G, pairs, mode=mode, strategy="plain_star", max_ctas=19)
+    assert lane["block_threads"] == 1024 and lane["ctas"] <= 19, lane
