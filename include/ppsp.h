@@ -80,7 +80,8 @@ enum {
     PPSP_BATCH_MULTI = 0,      /* Multi-BiDS: one search per query-graph vertex, shared  */
     PPSP_BATCH_PLAIN_STAR = 1, /* Plain*: every query its own pair of searches, all at once */
     PPSP_BATCH_PLAIN = 2,      /* Plain: one query at a time, each on one team of team_ctas
-                                  CTAs (default: the whole GPU)                           */
+                                  CTAs (default: the whole GPU, or, where the kernels over
+                                  adjacency blocks run, one CTA or a cluster of 2 to 8)   */
     PPSP_BATCH_SSSP = 3,       /* Plain-SSSP (Sec. 4.3): a single-source search from every
                                   query source; answers read from its distances          */
     PPSP_BATCH_VC = 4,         /* VC-SSSP (Sec. 4.3): single-source searches only from a
@@ -119,7 +120,8 @@ typedef struct {
     int32_t batch_strategy;  /* PPSP_BATCH_* (default MULTI)                                */
     int32_t block_threads;   /* 256, 512 or 1024 threads per CTA; 0 = auto: by the number of
                                 groups and the graph's degrees                             */
-    int32_t team_ctas;       /* CTAs cooperating on one small group (pair); 0 = auto        */
+    int32_t team_ctas;       /* CTAs cooperating on one small group (pair); 0 = auto (1:
+                                one CTA per group, all of one size)                         */
     int32_t big_team_ctas;   /* CTAs cooperating on one multi-search group; 0 = auto        */
     uint32_t dense_den;      /* frontier goes dense above (searches * n) / dense_den; 0=auto */
     int32_t want_paths;      /* 1: also return one shortest path per query (weights >= 1)   */

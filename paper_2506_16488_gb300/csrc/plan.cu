@@ -1008,7 +1008,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         bool all_pairs_pot = !tsize;  // BiD-A* pairs only
         for (u32 gi : small)
             all_pairs_pot = all_pairs_pot && P->groups[gi].mode == GM_BIDIR && P->searches[P->groups[gi].sbeg].pot;
-        if (!tsize && !o.want_paths && bb == 1024 && !small.empty()) {
+        if (!tsize && !o.want_paths && !o.team_ctas && bb == 1024 && !small.empty()) {
             double best = 0;
             for (u32 k = 1; k <= 8; k *= 2) {
                 int nteams = sms;
@@ -1037,7 +1037,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         }
         // The longest groups on more threads each, beside the rest.
         LongGroups lg;
-        if (all_pairs_pot && (bb == 1024 || !o.block_threads) && !o.max_ctas &&
+        if (all_pairs_pot && (bb == 1024 || !o.block_threads) && !o.max_ctas && !o.team_ctas &&
             strategy != PPSP_BATCH_PLAIN && small.size() > 1) {
             const u32 per_sm = bb == 512 ? 2 : 1;
             std::vector<double> us[4];

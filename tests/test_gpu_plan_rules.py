@@ -36,3 +36,14 @@ def test_one_group_at_a_time_gets_whole_ctas(road, mode):
     assert many["block_threads"] == 1024 and many["cluster"] == few["cluster"], (few, many)
     lane = shape_of(G, pairs, mode=mode, strategy="plain_star", max_ctas=19)
     assert lane["block_threads"] == 1024 and lane["ctas"] <= 19, lane
+
+
+def test_team_of_one_cta_is_one_cta(road):
+    g, G = road
+    pairs = random_pairs(g, 400, 63)
+    auto = shape_of(G, pairs[:6], mode="et", strategy="plain_star")
+    assert auto["kernel"] == "clusters"
+    for mode in ("et", "bids", "bidastar"):
+        for k, strategy in ((6, "plain_star"), (6, "plain"), (400, "plain_star")):
+            s = shape_of(G, pairs[:k], mode=mode, strategy=strategy, team_ctas=1)
+            assert s["cluster"] == 1 and s["long_groups"] == 0 and s["ctas"] == s["teams"], (mode, k, s)
