@@ -289,6 +289,12 @@ std::vector<SrcDir> sssp_sources(int strategy, bool directed, const std::vector<
     return src;
 }
 
+// Time of a group of 512 threads beside another one on the SM, over that of
+// 1,024 threads alone, for all groups and the longest: 1,000 BiD-A* queries on
+// the 1024^2 road graph 1.47, the 32 longest of them 1.59; one-directional A*
+// on 500^2 1.35 and 1.40.
+constexpr double GROUP_512 = 1.45, LONG_512 = 1.6;
+
 // Bucketed kernel: shared-memory entries per bucket.  The ring (64 buckets of
 // 8- or 16-byte entries) takes 128 KB of an SM, whatever the CTAs' size.
 u32 bucket_cap(int block, int dist_bits) { return (u32)block / 4 / (dist_bits == 64 ? 2 : 1); }
@@ -308,18 +314,15 @@ u32 bucket_cap(u32 ring_entries, int block, int dist_bits) {
 // 2.1 to 2.4).  Searches with a potential take more steps per H the longer the
 // query (BiD-A*: 1.29 at a mean H of 483, 1.5 at 1974).
 // busy: what a cluster's entry costs more, over one CTA's.
-double bucket_group_us(u32 mode, bool pot, double H, double n, u32 cl, double busy = 0.0) {
+// threads: of a CTA; an entry takes LONG_512 times as long with half of them.
+double bucket_group_us(u32 mode, bool pot, double H, double n, u32 cl, double busy = 0.0, int threads = 1024) {
     const double c = mode == GM_BIDIR ? (pot ? 0.3 : 1.05) : mode == GM_ASTAR ? 0.5 : 2.2;
     const double steps = 1.2 * H * (pot ? std::pow(std::max(H, 1.0) / 500.0, 0.15) : 1.0) + 20.0;
     const double entries = std::min(c * H, 2.0 * n / steps);
-    return steps * (2.2 + (cl > 1 ? 2.0 : 0.0) + 0.0105 * entries * (1.0 / cl + (cl > 1 ? busy : 0.0)));
+    const double entry = 0.0105 * std::pow(LONG_512, std::log2(1024.0 / threads));
+    return steps * (2.2 + (cl > 1 ? 2.0 : 0.0) + entry * entries * (1.0 / cl + (cl > 1 ? busy : 0.0)));
 }
 
-// Time of a group of 512 threads beside another one on the SM, over that of
-// 1,024 threads alone, for all groups and the longest: 1,000 BiD-A* queries on
-// the 1024^2 road graph 1.47, the 32 longest of them 1.59; one-directional A*
-// on 500^2 1.35 and 1.40.
-constexpr double GROUP_512 = 1.45, LONG_512 = 1.6;
 // What a cluster's entry costs more while the other SMs are busy, over one
 // CTA's entry: 256 BiD-A* queries on the 4096^2 graph, the longest on four CTAs
 // 83 ms where one takes 105.
@@ -998,17 +1001,18 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         // A cluster of CTAs per group where there are too few groups for the
         // SMs and their steps are large, or the longest groups would outlast
         // the rest: the smallest estimated time, by a tenth at least.
-        auto group_us = [&](u32 gi, u32 k, double busy = 0.0) {
+        auto group_us = [&](u32 gi, u32 k, double busy = 0.0, int threads = 1024) {
             const GroupDev& G = P->groups[gi];
             const double H = g->info.has_coords ? gdist[gi] : std::sqrt((double)n) / 2;
-            return bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k, busy);
+            return bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k, busy, threads);
         };
         u32 cl = 1, ncl = 0;
         double alone = 0;  // estimated time of the groups in one launch
         bool all_pairs_pot = !tsize;  // BiD-A* pairs only
         for (u32 gi : small)
             all_pairs_pot = all_pairs_pot && P->groups[gi].mode == GM_BIDIR && P->searches[P->groups[gi].sbeg].pot;
-        if (!tsize && !o.want_paths && !o.team_ctas && bb == 1024 && !small.empty()) {
+        if (!tsize && !o.want_paths && !o.team_ctas && bb >= 512 &&
+            (bb == 1024 || o.block_threads) && !small.empty()) {
             double best = 0;
             for (u32 k = 1; k <= 8; k *= 2) {
                 int nteams = sms;
@@ -1021,7 +1025,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 if (nteams < 1) break;
                 double sum = 0, most = 0;
                 for (u32 gi : small) {
-                    const double us = group_us(gi, k, all_pairs_pot && small.size() * k > (size_t)sms ? CLUSTER_BUSY : 0.0);
+                    const double us = group_us(gi, k, all_pairs_pot && small.size() * k > (size_t)sms ? CLUSTER_BUSY : 0.0, bb);
                     sum += us;
                     most = std::max(most, us);
                 }

@@ -47,3 +47,14 @@ def test_team_of_one_cta_is_one_cta(road):
         for k, strategy in ((6, "plain_star"), (6, "plain"), (400, "plain_star")):
             s = shape_of(G, pairs[:k], mode=mode, strategy=strategy, team_ctas=1)
             assert s["cluster"] == 1 and s["long_groups"] == 0 and s["ctas"] == s["teams"], (mode, k, s)
+
+
+def test_clusters_of_512_threads(road):
+    g, G = road
+    pairs = random_pairs(g, 6, 64)
+    want = oracle.pairs(g.offsets, g.targets, g.weights, pairs)
+    for bits in (32, 64):
+        s = shape_of(G, pairs, mode="et", strategy="plain_star", block_threads=512, dist_bits=bits)
+        assert s["kernel"] == "clusters" and s["block_threads"] == 512, s
+        got = G.batch(pairs, mode="et", strategy="plain_star", block_threads=512, dist_bits=bits)
+        assert np.array_equal(got, want)
