@@ -964,6 +964,13 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         const bool one = !plain && (o.team_ctas == 1 || 2 * P->groups.size() > grid_max);
         bucket = blocks_pay(g, all_bidir, one, tsize == 0, ctas, (u32)sms);
     }
+    // CTAs of 256 threads take four times as long for a step of a few hundred
+    // entries, and no cluster of them is compiled: few searches without a
+    // potential share the queue path (BiDS, 24 pairs on a 700^2 road graph 34.5 ms
+    // on one CTA each, 9.4 there; BiD-A* 8.2 against 23).
+    if (bucket && o.block_threads == 256 && !o.team_ctas && !tsize &&
+        (strategy == PPSP_BATCH_PLAIN || 2 * P->groups.size() <= grid_max))
+        for (u32 gi : small) bucket = bucket && (P->groups[gi].mode == GM_ASTAR || P->searches[P->groups[gi].sbeg].pot != 0);
     // An explicit increment far above the best one makes few steps of many
     // thousand entries, which a large team shares better: few groups with one
     // go to the queue path, as all did before.  One BiD-A* query at a time on

@@ -58,3 +58,14 @@ def test_clusters_of_512_threads(road):
         assert s["kernel"] == "clusters" and s["block_threads"] == 512, s
         got = G.batch(pairs, mode="et", strategy="plain_star", block_threads=512, dist_bits=bits)
         assert np.array_equal(got, want)
+
+
+def test_ctas_of_256_threads(road):
+    g, G = road
+    pairs = random_pairs(g, 24, 76)
+    want = oracle.pairs(g.offsets, g.targets, g.weights, pairs)
+    for mode, kernel in (("bids", "general"), ("et", "general"), ("bidastar", "bucket"), ("astar", "bucket")):
+        for k, strategy in ((24, "plain_star"), (1, "plain")):
+            s = shape_of(G, pairs[:k], mode=mode, strategy=strategy, block_threads=256)
+            assert (s["kernel"], s["block_threads"]) == (kernel, 256), (mode, s)
+        assert np.array_equal(G.batch(pairs, mode=mode, strategy="plain_star", block_threads=256), want), mode
