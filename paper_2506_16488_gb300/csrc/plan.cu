@@ -983,6 +983,21 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
                 div = std::max(div, astar_divisor(P->groups[gi].mode == GM_BIDIR, gdist[gi]) / 1.5);
         if ((double)o.delta * div > g->info.w_mean) bucket = false;
     }
+    // Whether `count` slots are idle in the graph's pool or fit half of the
+    // memory that is free now.
+    auto slots_free = [&](const SlotCaps& sc, u64 count) {
+        u64 idle = 0;
+        for (auto it = g->idle.lower_bound(SlotKey{o.dist_bits, sc.flat_cap, 0, 0, false});
+             it != g->idle.end() && it->first.dist_bits == o.dist_bits && it->first.flat_cap <= 2 * sc.flat_cap + 4096; ++it)
+            idle += it->first.qcap >= sc.qcap && it->first.tcap >= sc.tcap;
+        if (idle >= count) return true;
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+            cudaGetLastError();
+            return true;
+        }
+        return (count - idle) * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap) <= free_b / 2;
+    };
     if (bucket) {
         EngineKind kind = tsize ? ENGINE_BUCKET_TEAMS : ENGINE_BUCKET;
         const u64 want = small.size() + (u64)tsize * big.size();  // CTAs that run everything at once
@@ -1001,7 +1016,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             const u64 two = 2ull * sms * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap);
             const bool both = strategy != PPSP_BATCH_PLAIN && want > 4 * (u64)sms &&
                               (!o.max_ctas || 2 * (u64)o.max_ctas > 3 * (u64)sms);
-            bb = (both && two <= g->device_mem / 4) ? 512 : 1024;
+            bb = (both && two <= g->device_mem / 4 && slots_free(sc, 2ull * sms)) ? 512 : 1024;
         }
         const u32 cap = bucket_cap(o.ring_entries, bb, o.dist_bits);
         const u32 long_cap = bucket_cap(o.ring_entries, 1024, o.dist_bits);
@@ -1073,7 +1088,9 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             if (alone > 0) lg = long_groups(us, most, (u32)sms, per_sm, alone);
             const SlotCaps sc = slot_caps(small_range, o.frontier, false);
             const u64 slots = lg.teams + std::min<u64>(small.size() - lg.groups, (u64)per_sm * sms);
-            if (slots * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap) > g->device_mem / 2) lg = LongGroups();
+            if (lg.groups && (slots * slot_alloc_bytes(o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap) > g->device_mem / 2 ||
+                              !slots_free(sc, slots)))
+                lg = LongGroups();
             if (lg.groups) {
                 kind = ENGINE_BUCKET;
                 cl = 1;
@@ -1184,9 +1201,9 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         const SlotCaps sc = slot_caps(range_q[teams[t].queue], o.frontier, teams[t].size == grid);
         Slot* s = nullptr;
         st = slot_acquire(g, o.dist_bits, sc.flat_cap, sc.qcap, sc.tcap, P->memo, P->stream, &s);
-        if (st == PPSP_ERR_OOM && P->args.long_ctas && t > P->args.long_ctas / P->args.cluster) {
-            // two launches hold more slots than one would: run with fewer teams
-            grid -= (u32)teams.size() - t;
+        if (st == PPSP_ERR_OOM && P->kind >= ENGINE_BUCKET && teams[t].queue == 1 && t > 0 && teams[t - 1].queue == 1) {
+            // the teams of a queue take its groups in turn: run with fewer
+            grid = P->team_first[t];
             P->grid = grid;
             P->cta_team.resize(grid);
             P->team_first.resize(t);

@@ -69,3 +69,22 @@ def test_ctas_of_256_threads(road):
             s = shape_of(G, pairs[:k], mode=mode, strategy=strategy, block_threads=256)
             assert (s["kernel"], s["block_threads"]) == (kernel, 256), (mode, s)
         assert np.array_equal(G.batch(pairs, mode=mode, strategy="plain_star", block_threads=256), want), mode
+
+
+def test_fewer_teams_where_memory_is_short():
+    g = road_like_graph(900, seed=65)
+    pairs = random_pairs(g, 900, 66)
+    want = oracle.pairs(g.offsets, g.targets, g.weights, pairs[:30])
+    with ppsp.Graph.from_csr(g) as G:
+        per = G.slot_bytes(2, 32)
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        for room in (40, 170):  # slots that fit beside the caller's tensors
+            held = torch.empty(free - room * per - (64 << 20), dtype=torch.uint8, device="cuda")
+            try:
+                for mode in ("bids", "bidastar"):
+                    got = G.batch(pairs, mode=mode, strategy="plain_star")
+                    assert np.array_equal(got[:30], want), mode
+            finally:
+                del held
+                torch.cuda.empty_cache()
