@@ -337,10 +337,13 @@ SlotLayout slot_layout(int dist_bits, u64 flat_cap, u32 qcap, u32 tcap, bool mem
     const u64 words = (flat_cap + 31) / 32;
     auto al = [](u64 x) { return (x + 255) & ~255ull; };
     SlotLayout L;
-    // entries beyond the ring's shared-memory ones, split between its buckets:
-    // at least 4,096 each, so that a coarse increment on a small graph does
-    // not spill (a spilled bucket costs a scan of the slot's bitmap)
-    L.ocap = std::max<u64>(64 * 4096, flat_cap / 4) / 64 * 64;
+    // entries beyond the ring's shared-memory ones, split between its 64
+    // buckets: 4,096 each, so that a coarse increment does not spill (a spilled
+    // bucket costs a scan of the slot's bitmap), or, on small graphs, whose bitmap
+    // is quickly scanned, a 64th of the slot's distances, so that slots stay in
+    // proportion to the graph (a 64^2 grid: 2.2 MB a slot with 4,096 always, 0.2
+    // MB so; 300 ET pairs on 64^2, 128^2, 256^2 at any increment within 1%)
+    L.ocap = std::max<u64>({64 * 128, flat_cap / 4, std::min<u64>(64 * 4096, flat_cap)}) / 64 * 64;
     L.b_dist = al(flat_cap * W);
     L.b_bm = al(words * 4);
     L.b_q = al((u64)qcap * 4);

@@ -88,3 +88,15 @@ def test_fewer_teams_where_memory_is_short():
             finally:
                 del held
                 torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("side", [64, 128, 256, 512])
+def test_slots_in_proportion_to_the_graph(side):
+    g = grid_graph(side, seed=67)
+    with ppsp.Graph.from_csr(g) as G:
+        assert G.slot_bytes(2, 32) <= 40 * 2 * g.n and G.slot_bytes(2, 64) <= 60 * 2 * g.n
+        pairs = random_pairs(g, 300, 68)
+        want = oracle.pairs(g.offsets, g.targets, g.weights, pairs)
+        for delta in (0, 5000, 1 << 40):  # coarse increments overflow the buckets
+            got = G.batch(pairs, mode="et", strategy="plain_star", delta=delta, team_ctas=1)
+            assert np.array_equal(got, want), delta
