@@ -277,45 +277,52 @@ static Growth graph_growth(u64 n, const u64* off, const u32* tgt) {
     return count[GROWTH_RANDOM] > count[GROWTH_WIDE] ? GROWTH_RANDOM : GROWTH_WIDE;
 }
 
-bool HostWorkspace::reserve(size_t dev_need, size_t host_need) {
-    // sizes are rounded up, so that calls of about the same size allocate once
-    auto up = [](size_t x) { return (x + (x >> 2) + 65535) & ~(size_t)65535; };
+bool HostWorkspace::reserve(size_t dev_need, size_t host_need, cudaStream_t stream) {
     if (dev_need > dev_bytes) {
-        cudaFree(dev);
+        // rounded up, so that calls of about the same size allocate once
+        const size_t bytes = (dev_need + (dev_need >> 2) + 65535) & ~(size_t)65535;
+        if (dev) cudaFreeAsync(dev, stream);
         dev = nullptr;
         dev_bytes = 0;
-        if (cudaMalloc(&dev, up(dev_need)) != cudaSuccess) {
+        if (cudaMallocAsync(&dev, bytes, stream) != cudaSuccess) {
             dev = nullptr;
             cudaGetLastError();
             return false;
         }
-        dev_bytes = up(dev_need);
+        dev_bytes = bytes;
     }
-    if (host_need > host_bytes) {
-        cudaFreeHost(host);
-        host = nullptr;
-        host_bytes = 0;
-        if (cudaHostAlloc((void**)&host, up(host_need), cudaHostAllocDefault) != cudaSuccess) {
-            host = nullptr;
-            cudaGetLastError();
-            return false;
-        }
-        host_bytes = up(host_need);
+    if (host_need <= HOST_PINNED && !pinned &&
+        cudaHostAlloc((void**)&pinned, HOST_PINNED, cudaHostAllocDefault) != cudaSuccess) {
+        pinned = nullptr;
+        cudaGetLastError();
+    }
+    if (host_need <= HOST_PINNED && pinned) {
+        host = pinned;
+    } else {
+        if (pageable.size() < host_need) pageable.resize(host_need);
+        host = pageable.data();
     }
     return true;
 }
 
 void HostWorkspace::release() {
     cudaFree(dev);
-    cudaFreeHost(host);
+    cudaFreeHost(pinned);
     cudaGetLastError();
     dev = nullptr;
-    host = nullptr;
-    dev_bytes = host_bytes = 0;
+    pinned = host = nullptr;
+    dev_bytes = 0;
+    std::vector<char>().swap(pageable);
 }
 
-void HostWorkspace::trim() {
-    if (dev_bytes > HOST_KEEP || host_bytes > HOST_KEEP) release();
+void HostWorkspace::trim(cudaStream_t stream) {
+    if (dev_bytes > HOST_KEEP) {
+        cudaFreeAsync(dev, stream);
+        cudaGetLastError();
+        dev = nullptr;
+        dev_bytes = 0;
+    }
+    if (pageable.size() > HOST_KEEP) std::vector<char>().swap(pageable);
 }
 
 SlotCaps slot_caps(u64 range, int frontier, bool whole_gpu) {

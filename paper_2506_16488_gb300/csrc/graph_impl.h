@@ -13,19 +13,24 @@ namespace ppsp {
 
 // Memory of the calls that take host pairs and return host answers
 // (ppsp_query, ppsp_batch), kept by the graph between calls: the device arena
-// of the call's plan, and page-locked copies of what goes up and comes back.
-// A call holds the graph's lock until its work on its stream has ended, so one
-// call at a time uses it, whatever the stream.
+// of the call's plan, and host copies of what goes up and comes back.  A call
+// holds the graph's lock until its work on its stream has ended, so one call at
+// a time uses it, whatever the stream.  No call waits for another stream: the
+// arena grows in the stream-ordered pool, and the page-locked copies are
+// HOST_PINNED bytes allocated once, beyond which a call's copies are pageable
+// (cudaFree and cudaFreeHost wait for the whole device: a call whose workspace
+// grew took as long as the 967 ms of work on another stream, now 0.7 ms).
 struct HostWorkspace {
     void* dev = nullptr;
     size_t dev_bytes = 0;
-    char* host = nullptr;
-    size_t host_bytes = 0;
-    bool reserve(size_t dev_need, size_t host_need);
-    void trim();     // give back what a large call left (HOST_KEEP at most stays)
+    char* pinned = nullptr;
+    std::vector<char> pageable;
+    char* host = nullptr;  // pinned or pageable
+    bool reserve(size_t dev_need, size_t host_need, cudaStream_t stream);
+    void trim(cudaStream_t stream);  // give back what a large call left (HOST_KEEP at most stays)
     void release();
 };
-constexpr size_t HOST_KEEP = 64ull << 20;
+constexpr size_t HOST_KEEP = 64ull << 20, HOST_PINNED = 4ull << 20;
 
 // How fast a graph's neighbourhoods grow (graph_growth).
 enum Growth {

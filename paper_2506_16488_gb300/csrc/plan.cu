@@ -1257,7 +1257,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
     P->arena_bytes = off;
     const size_t up_bytes = host_call ? o_run + P->runstate_bytes : static_bytes;
     cudaError_t ce = cudaSuccess;
-    if (host_call && g->ws.reserve(P->arena_bytes, std::max(up_bytes, P->back_bytes))) {
+    if (host_call && g->ws.reserve(P->arena_bytes, std::max(up_bytes, P->back_bytes), P->stream)) {
         P->host_call = true;
         P->d_arena = g->ws.dev;
     } else if (host_call) {
@@ -1683,7 +1683,10 @@ static ppsp_status run_host(ppsp_graph* g, const uint32_t* pairs, uint64_t k, co
         for (u64 q = 0; q < k; ++q) caps[q] = hp->offsets ? hp->offsets[q + 1] - hp->offsets[q] : hp->single_cap;
     }
     ppsp_status st = plan_create_impl(g, pairs, k, opt, single, &P, hp ? caps.data() : nullptr, true);
-    if (st != PPSP_OK) return st;
+    if (st != PPSP_OK) {
+        g->ws.trim(opt ? (cudaStream_t)opt->stream : nullptr);
+        return st;
+    }
     st = plan_launch_direct(P, nullptr);
     if (st == PPSP_OK)
         st = host_finish(P, counters, dists_out);
@@ -1737,7 +1740,7 @@ static ppsp_status run_host(ppsp_graph* g, const uint32_t* pairs, uint64_t k, co
         if (st == PPSP_OK && small) st = PPSP_ERR_BUFFER_TOO_SMALL;
     }
     plan_free(P);
-    g->ws.trim();
+    g->ws.trim(opt ? (cudaStream_t)opt->stream : nullptr);
     return st;
 }
 

@@ -100,3 +100,25 @@ def test_slots_in_proportion_to_the_graph(side):
         for delta in (0, 5000, 1 << 40):  # coarse increments overflow the buckets
             got = G.batch(pairs, mode="et", strategy="plain_star", delta=delta, team_ctas=1)
             assert np.array_equal(got, want), delta
+
+
+def test_host_calls_do_not_wait_for_other_streams():
+    g = grid_graph(64, seed=74)
+    pair = random_pairs(g, 1, 75)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    with ppsp.Graph.from_csr(g) as G, ppsp.Graph.from_csr(g) as H:
+        # the search memory of one team is there (its first allocation is not the question)
+        with G.plan(pair, mode="bids", strategy="plain_star", stream=mine.cuda_stream) as p:
+            p.run(torch.zeros(1, dtype=torch.int64, device="cuda").data_ptr())
+            p.sync()
+        want = G.query(*pair[0].tolist())
+        H.query(*pair[0].tolist())
+        done = torch.cuda.Event()
+        with torch.cuda.stream(other):
+            torch.cuda._sleep(4_000_000_000)  # about two seconds
+        done.record(other)
+        for k in (1, 2000, 20000, 100000, 400000, 1):
+            got = G.batch(np.tile(pair, (k, 1)), mode="bids", strategy="plain_star", stream=mine.cuda_stream)
+            assert got.shape == (k,) and (got == want).all()
+            assert not done.query(), f"the call with {k} pairs waited for another stream"
+        done.synchronize()
