@@ -126,8 +126,9 @@ typedef struct {
     uint32_t dense_den;      /* frontier goes dense above (searches * n) / dense_den; 0=auto */
     int32_t want_paths;      /* 1: also return one shortest path per query (weights >= 1)   */
     int32_t max_ctas;        /* cap on resident CTAs used (0 = all that fit)               */
-    uint64_t spin_limit;     /* iterations of a device-side wait before PPSP_ERR_TIMEOUT;
-                                0 = default (about a few seconds)                          */
+    uint64_t spin_limit;     /* iterations of a device-side wait without a step of the CTAs
+                                waited for before PPSP_ERR_TIMEOUT; 0 = default (about a few
+                                seconds)                                                   */
     void* stream;            /* cudaStream_t to run on; NULL = the legacy default stream    */
     uint32_t debug_flags;    /* test hooks, 0 in normal use (PPSP_DEBUG_*)                  */
     uint32_t cuda_graph;     /* plans: 1 = capture the launches of ppsp_plan_run into a CUDA

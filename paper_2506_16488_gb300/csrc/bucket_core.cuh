@@ -931,6 +931,7 @@ __device__ __forceinline__ bool bk_group(const EngineArgs& a, const TeamCtx& tc,
         if (t < 32) bk_decide<D, KIND, CL>(a, c, sm, fresh, par);
         __syncthreads();
         const u32 what = sm.what;
+        if (KIND == BK_MULTI && t == 0) atomicAdd(&tc.ts->progress, 1u);  // the searches that are done wait
         if (what == 3) break;
         c.cur_lo = (u32)sm.cur;
         c.kc = sm.key_off - (i64)sm.curkey;
@@ -1048,7 +1049,7 @@ __global__ void __launch_bounds__(B, (BucketMinBlocks<B>::value)) bucket_kernel(
     tc.ts = a.tstate + tc.team;
     tc.global_bar = RUN == BK_TEAMS && tc.size > 1;
     tc.expect = tc.size;
-    tc.wait_shift = 4;
+    tc.watch = true;
     const u32 qid = a.team_queue[tc.team];
     if (RUN != BK_TEAMS && a.part == 1) cudaTriggerProgrammaticLaunchCompletion();
     if (threadIdx.x == 0) {

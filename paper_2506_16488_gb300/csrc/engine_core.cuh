@@ -135,7 +135,7 @@ struct TeamCtx {
     TeamState* ts;
     bool global_bar;  // size > 1 or a test hook forces the global path
     u32 expect;       // arrivals that release the barrier
-    u32 wait_shift = 0;  // spins allowed: the limit times 2^wait_shift (waits for a whole search)
+    bool watch = false;  // waits for whole searches: the limit is between two of their steps
 };
 
 static __device__ bool team_sync(const TeamCtx& tc, const EngineArgs& a, u32* s_flag) {
@@ -152,12 +152,19 @@ static __device__ bool team_sync(const TeamCtx& tc, const EngineArgs& a, u32* s_
             atomicAdd(&tc.ts->bar_gen, 1u);
         } else {
             u64 it = 0;
+            u32 seen = tc.watch ? ld_volatile(&tc.ts->progress) : 0u;
             while (ld_volatile(&tc.ts->bar_gen) == gen) {
                 if (ld_volatile(a.err) != 0) {  // another CTA failed: leave
                     ok = 0;
                     break;
                 }
-                if (++it >> tc.wait_shift > a.spin_limit) {
+                if (++it > a.spin_limit) {
+                    const u32 now = tc.watch ? ld_volatile(&tc.ts->progress) : seen;
+                    if (now != seen) {
+                        seen = now;
+                        it = 0;
+                        continue;
+                    }
                     atomicOr(a.err, ERRB_TIMEOUT);
                     ok = 0;
                     break;

@@ -153,7 +153,8 @@ struct TeamState {
     u32 bar_count;
     u32 bar_gen;
     u32 group;
-    u32 pad[29];          // one 128-byte line per team
+    u32 progress;         // steps of the team's searches (Multi-BiDS, one CTA each)
+    u32 pad[28];          // one 128-byte line per team
 };
 
 struct EngineCounters {

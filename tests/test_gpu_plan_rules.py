@@ -122,3 +122,13 @@ def test_host_calls_do_not_wait_for_other_streams():
             assert got.shape == (k,) and (got == want).all()
             assert not done.query(), f"the call with {k} pairs waited for another stream"
         done.synchronize()
+
+
+@pytest.mark.parametrize("limit", [1 << 8, 1 << 10])
+def test_spin_limit_counts_from_a_search_s_last_step(road, limit):
+    g, G = road
+    pairs = clique_pairs(g, 8, 73)
+    want = oracle.pairs(g.offsets, g.targets, g.weights, pairs)
+    assert shape_of(G, pairs, mode="bids", strategy="multi")["kernel"] == "bucket_teams"
+    for _ in range(3):
+        assert np.array_equal(G.batch(pairs, mode="bids", strategy="multi", spin_limit=limit), want)
