@@ -378,7 +378,11 @@ LongGroups long_groups(const std::vector<double> us[4], const u32 max_teams[4], 
 // one.  H: heuristic distance in mean edge weights.  One-directional A*, six
 // random pairs, w/4, w/8, w/16: 512^2 (H about 265) 12.2, 6.6, 11.3 ms; 1024^2
 // 57, 13.7, 16.1; 2048^2 1037, 224, 60.  BiD-A*, 1,000 pairs on 1024^2, w/4,
-// w/8, w/16, w/32: 139, 25.9, 16.2, 19.9 ms.
+// w/8, w/16, w/32: 139, 25.9, 16.2, 19.9 ms.  On graphs that grow faster than the
+// plane paths have few hops and one mean weight stays, but for one-directional
+// A* on one CTA per group (random graph of 2^20 vertices with coordinates, one
+// mean weight / this: A* 8 queries one at a time 4.7 / 7.5 ms, 24 pairs 12.9 /
+// 25.9, 200 906 / 181; BiD-A* 1,000 pairs 2.0 / 2.2).
 double astar_divisor(bool bidir, double H) {
     return bidir ? std::min(32.0, std::max(8.0, H / 32.0)) : std::min(32.0, std::max(6.0, H / 64.0));
 }
@@ -782,7 +786,7 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         }
         gwork[gi] = work;
         gdist[gi] = (double)*std::max_element(hmax.begin(), hmax.end()) / std::max(1e-9, g->info.w_mean);
-        if (o.delta == 0 && g->delta_model[o.mode] == nullptr &&
+        if (o.delta == 0 && g->delta_model[o.mode] == nullptr && g->growth == GROWTH_PLANE &&
             (G.mode == GM_ASTAR || (G.mode == GM_BIDIR && P->searches[G.sbeg].pot == 1)))
             G.delta = std::max<u64>(1, (u64)std::llround((double)delta / astar_divisor(bidir, gdist[gi])));
         P->groups.push_back(G);
@@ -1173,6 +1177,11 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
             }
         }
     }
+    if (o.delta == 0 && g->delta_model[o.mode] == nullptr && g->growth != GROWTH_PLANE && all_single(teams))
+        for (u32 gi = 0; gi < NG; ++gi)
+            if (P->groups[gi].mode == GM_ASTAR)
+                P->groups[gi].delta =
+                    std::max<u64>(1, (u64)std::llround((double)delta / astar_divisor(false, gdist[gi])));
     P->grid = grid;
     u32 first = 0;
     for (u32 t = 0; t < teams.size(); ++t) {

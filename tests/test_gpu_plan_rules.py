@@ -132,3 +132,25 @@ def test_spin_limit_counts_from_a_search_s_last_step(road, limit):
     assert shape_of(G, pairs, mode="bids", strategy="multi")["kernel"] == "bucket_teams"
     for _ in range(3):
         assert np.array_equal(G.batch(pairs, mode="bids", strategy="multi", spin_limit=limit), want)
+
+
+def test_astar_increment_where_paths_have_few_hops():
+    rng = np.random.default_rng(71)
+    n = 1 << 17
+    u, v = rng.integers(0, n, (2, 5 * n // 2))
+    lo, hi = np.minimum(u, v), np.maximum(u, v)
+    key = np.unique((lo * n + hi)[lo != hi])
+    lo, hi = key // n, key % n
+    xy = rng.uniform(0, 1000, (n, 2)).astype(np.float32)
+    w = (10 * np.sqrt(((xy[lo].astype(float) - xy[hi]) ** 2).sum(1)) + rng.integers(10, 1000, lo.size)).astype(np.uint32)
+    off, tgt, wt = csr_from_undirected(n, lo, hi, w)
+    g = CSRGraph(n=n, offsets=off, targets=tgt, weights=wt, coords=xy,
+                 lcc=np.flatnonzero(np.diff(off.astype(np.int64)) >= 2).astype(np.uint32))
+    pairs = random_pairs(g, 8, 72)
+    want = oracle.pairs(g.offsets, g.targets, g.weights, pairs)
+    with ppsp.Graph.from_csr(g) as G:
+        mean = int(round(G.info()["w_mean"]))
+        for mode in ("astar", "bidastar"):
+            got, auto = G.batch(pairs, mode=mode, strategy="plain_star", return_counters=True)
+            _, one = G.batch(pairs, mode=mode, strategy="plain_star", delta=mean, return_counters=True)
+            assert np.array_equal(got, want) and auto["rounds"] < 1.5 * one["rounds"], (mode, auto, one)
