@@ -1029,14 +1029,18 @@ static ppsp_status plan_create_impl(ppsp_graph* g, const uint32_t* pairs, uint64
         // the rest: the smallest estimated time, by a tenth at least.
         auto group_us = [&](u32 gi, u32 k, double busy = 0.0, int threads = 1024) {
             const GroupDev& G = P->groups[gi];
-            const double H = g->info.has_coords ? gdist[gi] : std::sqrt((double)n) / 2;
-            return bucket_group_us(G.mode, P->searches[G.sbeg].pot != 0, H, (double)n, k, busy, threads);
+            // without a potential on a scale (no coordinates, or none that the
+            // weights allow) the length of a query of a square grid
+            const bool scaled = g->info.has_coords && g->pot_scale > 0.0;
+            const double H = scaled ? gdist[gi] : std::sqrt((double)n) / 2;
+            const u32 mode = !scaled && G.mode == GM_ASTAR ? (u32)GM_ET : G.mode;
+            return bucket_group_us(mode, scaled && P->searches[G.sbeg].pot != 0, H, (double)n, k, busy, threads);
         };
         u32 cl = 1, ncl = 0;
         double alone = 0;  // estimated time of the groups in one launch
         bool all_pairs_pot = !tsize;  // BiD-A* pairs only
         for (u32 gi : small)
-            all_pairs_pot = all_pairs_pot && P->groups[gi].mode == GM_BIDIR && P->searches[P->groups[gi].sbeg].pot;
+            all_pairs_pot = all_pairs_pot && P->groups[gi].mode == GM_BIDIR && P->searches[P->groups[gi].sbeg].pot && g->pot_scale > 0.0;
         if (!tsize && !o.want_paths && !o.team_ctas && bb >= 512 &&
             (bb == 1024 || o.block_threads) && !small.empty()) {
             double best = 0;

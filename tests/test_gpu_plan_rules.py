@@ -154,3 +154,19 @@ def test_astar_increment_where_paths_have_few_hops():
             got, auto = G.batch(pairs, mode=mode, strategy="plain_star", return_counters=True)
             _, one = G.batch(pairs, mode=mode, strategy="plain_star", delta=mean, return_counters=True)
             assert np.array_equal(got, want) and auto["rounds"] < 1.5 * one["rounds"], (mode, auto, one)
+
+
+def test_estimates_without_a_scaled_potential():
+    # one edge of weight 0 leaves no positive potential: lengths are not known
+    g = road_like_graph(700, seed=69)
+    u = np.repeat(np.arange(g.n), np.diff(g.offsets.astype(np.int64)))
+    w = g.weights.copy()
+    a, b = int(u[0]), int(g.targets[0])
+    w[((u == a) & (g.targets == b)) | ((u == b) & (g.targets == a))] = 0
+    pairs = random_pairs(g, 6, 70)
+    want = oracle.pairs(g.offsets, g.targets, w, pairs)
+    with ppsp.Graph(g.offsets, g.targets, w, g.coords) as G:
+        assert G.info()["potential_scale"] == 0.0
+        for mode in ("et", "astar"):
+            assert shape_of(G, pairs, mode=mode, strategy="plain_star")["kernel"] == "clusters", mode
+            assert np.array_equal(G.batch(pairs, mode=mode, strategy="plain_star"), want), mode
