@@ -1213,8 +1213,7 @@ static ppsp_status bucket_occ_t(int* bpsm, u32 ring_cap) {
 template <typename D, int RUN>
 static ppsp_status bucket_occ(int block_threads, u32 ring_cap, int* bpsm) {
     if (ring_cap < 1 || ring_cap > RING_CAP_MAX) return PPSP_ERR_INVALID_ARG;
-    if (RUN != BK_CLUSTERS && block_threads == 256)
-        return bucket_occ_t<D, RUN == BK_CLUSTERS ? 512 : 256, RUN>(bpsm, ring_cap);
+    if (block_threads == 256) return bucket_occ_t<D, 256, RUN>(bpsm, ring_cap);
     if (block_threads == 512) return bucket_occ_t<D, 512, RUN>(bpsm, ring_cap);
     if (block_threads == 1024) return bucket_occ_t<D, 1024, RUN>(bpsm, ring_cap);
     return PPSP_ERR_INVALID_ARG;
