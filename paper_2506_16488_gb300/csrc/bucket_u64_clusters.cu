@@ -7,7 +7,6 @@ ppsp_status launch_bucket_u64_clusters(const EngineArgs& a, int block_threads, u
     return bucket_launch<u64, BK_CLUSTERS>(a, block_threads, grid, stream);
 }
 
-
 ppsp_status resident_bucket_u64_clusters(int block_threads, u32 ring_cap, u32 cluster, int* clusters) {
     return bucket_clusters<u64>(block_threads, ring_cap, cluster, clusters);
 }

@@ -69,6 +69,26 @@ static void parallel_for(u64 n, F f) {
     for (auto& t : th) t.join();
 }
 
+// f over the rows of a CSR, in ranges of about as many edges each (the rows of a
+// power-law graph's first ids hold half of its edges).
+template <typename OFF, typename F>
+static void parallel_rows(u64 n, const OFF* off, F f) {
+    const u64 m = off[n];
+    unsigned nt = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+    if (m < (1u << 16)) nt = 1;
+    std::vector<std::thread> th;
+    u64 lo = 0;
+    for (unsigned k = 0; k < nt; ++k) {
+        const u64 hi = k + 1 == nt ? n : (u64)(std::upper_bound(off + lo, off + n, (OFF)(m * (k + 1) / nt)) - off);
+        if (nt == 1)
+            f(lo, hi);
+        else
+            th.emplace_back([=, &f]() { f(lo, hi); });
+        lo = hi;
+    }
+    for (auto& t : th) t.join();
+}
+
 // The certified integer potential (Sec. 3.3, Fact 3.1): choose c and F, round
 // P(v) = floor(p(v) * c * 2^F + 0.5), and check |P(u)-P(v)|^2 <= (2^F w)^2 on
 // every edge in exact integer arithmetic; shrink c until the check passes.
@@ -142,14 +162,14 @@ static void build_potential(ppsp_graph* g, const u64* off, const u32* tgt, const
 static bool check_symmetric(u64 n, const u64* off, const u32* tgt, const u32* w) {
     const u64 m = off[n];
     std::vector<u64> key(m);
-    parallel_for(n, [&](u64 lo, u64 hi, unsigned) {
+    parallel_rows(n, off, [&](u64 lo, u64 hi) {
         for (u64 u = lo; u < hi; ++u) {
             for (u64 e = off[u]; e < off[u + 1]; ++e) key[e] = ((u64)tgt[e] << 32) | w[e];
             std::sort(key.begin() + off[u], key.begin() + off[u + 1]);
         }
     });
     std::atomic<bool> ok(true);
-    parallel_for(n, [&](u64 lo, u64 hi, unsigned) {
+    parallel_rows(n, off, [&](u64 lo, u64 hi) {
         for (u64 u = lo; u < hi && ok.load(std::memory_order_relaxed); ++u)
             for (u64 e = off[u]; e < off[u + 1]; ++e) {
                 u64 v = tgt[e];
@@ -536,11 +556,11 @@ ppsp_status ppsp_graph_create(uint64_t n, uint64_t m, const uint64_t* offsets, c
     g->wsorted = m > BLOCK_MAX_DEG * n;
     g->growth = graph_growth(n, offsets, targets);
     auto sort_rows = [](u64 rows, const auto* off, uint2* ed) {
-        parallel_for(rows, [&](u64 lo, u64 hi, unsigned) {
+        auto key = [](const uint2& x) { return ((u64)x.y << 32) | x.x; };
+        parallel_rows(rows, off, [&](u64 lo, u64 hi) {
             for (u64 v = lo; v < hi; ++v)
-                std::sort(ed + off[v], ed + off[v + 1], [](const uint2& x, const uint2& y) {
-                    return x.y != y.y ? x.y < y.y : x.x < y.x;
-                });
+                std::sort(ed + off[v], ed + off[v + 1],
+                          [&](const uint2& x, const uint2& y) { return key(x) < key(y); });
         });
     };
     ppsp_graph_info& info = g->info;
