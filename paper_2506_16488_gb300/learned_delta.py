@@ -228,6 +228,96 @@ def _training_sets(mode: str, build: bool = True):
     return sets
 
 
+# ---- more graph shapes for a trained model ----
+def _undirected(n: int, u, v, w, coords=None):
+    from workloads import CSRGraph, csr_from_undirected
+
+    off, tgt, wt = csr_from_undirected(n, u, v, w)
+    return CSRGraph(n=n, offsets=off, targets=tgt, weights=wt, coords=coords,
+                    lcc=np.flatnonzero(np.diff(off.astype(np.int64)) >= 2).astype(np.uint32))
+
+
+def mesh_graph(side: int, seed: int, jitter: float = 0.3, longest: float = 3.0):
+    """A point in each of side^2 cells, joined to those of the eight neighbours
+    that are no farther than `longest` cells."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(side * side).reshape(side, side)
+    u = np.r_[i[:, :-1].ravel(), i[:-1].ravel(), i[:-1, :-1].ravel(), i[:-1, 1:].ravel()]
+    v = np.r_[i[:, 1:].ravel(), i[1:].ravel(), i[1:, 1:].ravel(), i[1:, :-1].ravel()]
+    xy = (np.stack([np.arange(side * side) % side, np.arange(side * side) // side], 1)
+          + rng.uniform(-jitter, jitter, (side * side, 2))).astype(np.float32)
+    length = np.sqrt(((xy[u].astype(np.float64) - xy[v]) ** 2).sum(1))
+    u, v, length = u[length <= longest], v[length <= longest], length[length <= longest]
+    return _undirected(side * side, u, v, np.maximum(1, np.ceil(1000 * length)).astype(np.uint32), xy)
+
+
+def sparse_graph(n: int, degree: float, ring: int, seed: int):
+    """Random edges of the given average degree over a ring lattice that joins
+    each vertex to the `ring` next ones; weights 1 .. 1000."""
+    rng = np.random.default_rng(seed)
+    u, v = rng.integers(0, n, (2, int(n * degree / 2)))
+    for k in range(1, ring + 1):
+        u, v = np.r_[u, np.arange(n)], np.r_[v, (np.arange(n) + k) % n]
+    lo, hi = np.minimum(u, v), np.maximum(u, v)
+    key = np.unique((lo * n + hi)[lo != hi])
+    return _undirected(n, key // n, key % n, rng.integers(1, 1001, key.size).astype(np.uint32))
+
+
+EXTENSION = ("mesh512", "scatter512", "scatter256", "random19", "smallworld19", "sparse_rmat17")
+
+
+def extension_sets() -> list:
+    """(name, graph, pairs, first grid point): shapes that the BiDS model was
+    not trained on and took for an RMAT's."""
+    from workloads import random_pairs, rmat_graph
+
+    sets = [("mesh512", mesh_graph(512, 9701), 9702, 0), ("scatter512", mesh_graph(512, 9703, 0.5, 1.7), 9704, 0),
+            ("scatter256", mesh_graph(256, 9705, 0.5, 1.7), 9706, 0), ("random19", sparse_graph(1 << 19, 5.0, 0, 9711), 9712, 0),
+            ("smallworld19", sparse_graph(1 << 19, 0.2, 2, 9721), 9722, 0),
+            ("sparse_rmat17", rmat_graph(17, seed=9731, edge_factor=3), 9732, -6)]
+    return [(name, g, random_pairs(g, 96, seed), start) for name, g, seed, start in sets]
+
+
+def extend(mode: str, model, sweeps_dir: str = WEIGHTS_DIR, epochs: int = 1500, log=print):
+    """Train `model` on for the extension sets (their sweeps in `sweeps_dir`,
+    see `sweep`) without changing what it answers on the sets it was trained on:
+    those take part with its own answers, also between and around them (mixtures
+    of two groups of one family, and other graph sizes), and the new sets with
+    their labels less the model's margin."""
+    rng = np.random.default_rng(1)
+    meta = json.load(open(os.path.join(WEIGHTS_DIR, f"delta_{mode}.json")))
+
+    def load(name):
+        return np.load(os.path.join(sweeps_dir, f"sweep_{mode}_{name}.npz"))
+
+    old = {s["set"]: load(s["set"])["feats"] for s in meta["sets"]}
+    power = [n for n in old if n.startswith("rmat")]
+    families = [np.concatenate([old[n] for n in old if n not in power]), np.concatenate([old[n] for n in power])]
+    keep = list(families)
+    for f in families:
+        a, b = f[rng.integers(0, len(f), (2, 4000))]
+        t = rng.random((4000, 1), dtype=np.float32)
+        keep.append(t * a + (1 - t) * b)
+        resized = f[rng.integers(0, len(f), 2000)].copy()
+        resized[:, 7:9] += rng.uniform(-5, 2, (2000, 1)).astype(np.float32)  # n and m together
+        keep.append(resized)
+    K = np.concatenate(keep).astype(np.float32)
+    K, _ = unit_copies(K, np.zeros(len(K), dtype=np.float32))
+    F, Y = [K], [model.predict(K)]
+    for name in EXTENSION:
+        d = load(name)
+        f, y = unit_copies(d["feats"], labels_from_times(d["times"]) - meta["margin"])
+        F += [f] * 8
+        Y += [y] * 8
+    before = Y[0]
+    tuned = ppsp.DeltaModel(model.params())
+    for lr in (2e-3, 5e-4, 1e-4):
+        loss = tuned.train(np.concatenate(F), np.concatenate(Y).astype(np.float32), epochs, lr)
+    log(json.dumps({"loss": loss, "kept": float(np.abs(tuned.predict(K) - before).mean()),
+                    "kept_max": float(np.abs(tuned.predict(K) - before).max())}))
+    return tuned
+
+
 def ceil_regret(times: np.ndarray, y_pred: np.ndarray, grid=GRID) -> float:
     """Like `regret`, but a prediction between two grid points is charged the
     time of the larger increment (the pessimistic side of the steep curve)."""
