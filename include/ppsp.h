@@ -119,7 +119,7 @@ typedef struct {
     int32_t layout;          /* PPSP_LAYOUT_* (default AUTO)                                */
     int32_t batch_strategy;  /* PPSP_BATCH_* (default MULTI)                                */
     int32_t block_threads;   /* 256, 512 or 1024 threads per CTA; 0 = auto: by the number of
-                                groups and the graph's degrees                             */
+                                groups that run at once and the graph's degrees            */
     int32_t team_ctas;       /* CTAs cooperating on one small group (pair); 0 = auto (1:
                                 one CTA per group, all of one size)                         */
     int32_t big_team_ctas;   /* CTAs cooperating on one multi-search group; 0 = auto        */
@@ -151,8 +151,8 @@ typedef struct {
                                 on one CTA and directed graphs ignore it.  Default 0         */
     uint32_t ring_entries;   /* groups with buckets in shared memory: entries per Delta-bucket
                                 of the frontier ring there, 1..256; 0 = default: 64 of 32
-                                buckets, or, on graphs of at most six adjacency entries per
-                                vertex, the CTA's threads / 4 (/ 8 with 64-bit distances) of
+                                buckets, or, in the kernels over adjacency blocks (see
+                                ppsp_graph_create), the CTA's threads / 4 (/ 8 with 64-bit distances) of
                                 64 buckets (there at most 223 with 64-bit distances, what
                                 shared memory holds).
                                 Larger buckets stay out of the global overflow region; a
@@ -224,11 +224,13 @@ const char* ppsp_last_error_detail(void);
  *            searches with a potential read instead of gathering the
  *            target's coordinates separately
  *            A graph of at most six adjacency entries per vertex (and fewer
- *            than 2^29 vertices) also gets one aligned block per vertex with its
- *            first four edges, and the rest of longer rows: 36n bytes or more,
- *            100n with coordinates, about twice that for a directed graph (none
- *            where they would take more than an eighth of the free device
- *            memory); device_bytes of ppsp_graph_info counts them
+ *            than 2^29 vertices) whose neighbourhoods grow as in the plane, or
+ *            with at most 4,096 vertices or 64 entries in a row, also gets one
+ *            aligned block per vertex with its first four edges, and the rest of
+ *            longer rows: 36n bytes or more, 100n with coordinates, about twice
+ *            that for a directed graph (none where they would take more than an
+ *            eighth of the free device memory); device_bytes of ppsp_graph_info
+ *            counts them
  *   flags    PPSP_UNDIRECTED: the CSR is symmetric with equal weights both ways
  *            (validated; the bidirectional modes search backwards on the same CSR).
  *            Without it the graph is directed: the library also keeps its
