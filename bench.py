@@ -710,7 +710,7 @@ def main():
     ap.add_argument("--duration", type=float, default=2.0, help="serving (config 5): seconds per rate")
     ap.add_argument("--lanes", type=int, default=8, help="serving (config 5): concurrent micro-batches")
     ap.add_argument("--lane-ctas", type=int, default=0, help="serving (config 5): CTAs per lane (0 = SMs / lanes)")
-    ap.add_argument("--team-ctas", type=int, default=1, help="serving (config 5): CTAs per query (0 = auto)")
+    ap.add_argument("--team-ctas", type=int, default=0, help="serving (config 5): CTAs per query (0 = auto)")
     args = ap.parse_args()
     if args.impl == "reference":
         run_reference(args)
